@@ -119,13 +119,16 @@ typedef struct {
   int tile_capacity;          /* distinct new spawned keys one annihilation tile holds on
                                  chip: 0 = default (128 per warp on the warp path, 64 for
                                  512-bit keys; 512 for
-                                 64/128-bit and 256 for 512-bit keys on the block path),
+                                 64/128-bit and 256 for 512-bit keys on the block path; 16
+                                 times that many survivors per 64 entries are ranked by
+                                 counting on the hash path),
                                  else a power of two in [64, default]; smaller values only
                                  send more buckets through the slower paths */
-  int annihilation;           /* annihilation kernel: 0 = default (one warp per
-                                 bucket), 1 = block tiles, 2 = one warp per bucket (large
-                                 or overflowing buckets go to block tiles on that path);
-                                 every choice gives the same walker list */
+  int annihilation;           /* annihilation kernel: 0 = default (flat hash table; one
+                                 warp per bucket for state_capacity >= 2^31), 1 = block
+                                 tiles, 2 = one warp per bucket (large or overflowing
+                                 buckets go to block tiles on that path); every choice
+                                 gives the same walker list */
   int excit_gen;              /* excitation generator (the paper's `excit_gen`): 0 = the
                                  system's own (HUBBARD and UEG uniform, MOLECULE heat-bath);
                                  1 = UEG proposal table (the learned proposal's table, see
@@ -181,7 +184,8 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
                                void* cuda_stream, hande_ctx** out);
 
 /* Advance n >= 0 iterations (asynchronous; one CUDA-graph launch per iteration).
- * Errors of an iteration surface at the next synchronising call.  Annihilation
+ * Errors of an iteration surface at the next synchronising call.  With
+ * annihilation 1 or 2 the annihilation
  * buckets are sized from the previous iteration's spawn and new-key counts; a
  * bucket that still receives more spawns than one warp takes is split into at
  * most 256 key sub-ranges of about a quarter tile each (splitters sampled from
@@ -242,7 +246,8 @@ typedef struct {
 } hande_tuning;
 
 /* Autotune the annihilation bucket size (expected spawns and new determinants
- * per bucket, 0.5 to 1.25 times the defaults) and the spawning kernel's grid
+ * per bucket, 0.5 to 1.25 times the defaults; the hash path has none and is
+ * unaffected) and the spawning kernel's grid
  * (one or two blocks per SM): time `iterations` iterations of each candidate
  * and keep the fastest.  The iterations are real (the run advances by
  * 16 x (iterations + 1)); the walker lists do not depend on the choice.  *out
@@ -256,9 +261,11 @@ typedef struct {
                                  32 bucket capacity */
   int64_t ndet;               /* current list length */
   int64_t natt, nspawn;       /* attempts and spawns of the last iteration */
-  int64_t nbuckets;           /* annihilation buckets of the last iteration */
+  int64_t nbuckets;           /* annihilation buckets of the last iteration (hash path:
+                                 groups of 64 main-list entries) */
   int64_t bucket_main;        /* main-list entries per bucket */
-  int64_t max_bucket_spawns;  /* largest number of spawns that fell in one bucket */
+  int64_t max_bucket_spawns;  /* largest number of spawns that fell in one bucket (hash
+                                 path: of new determinants that survived in one group) */
   int64_t tile_capacity;      /* distinct spawned keys one bucket can hold on chip */
   int64_t ncore;              /* deterministic-space size */
   int64_t launches_per_iteration; /* kernels one iteration launches (current settings) */

@@ -115,7 +115,8 @@ hande_status fork_all(hande_batch* b) {
 // group key: replicas whose iterations are the same kernels with the same
 // launch shapes
 bool same_group(const Engine& a, const Engine& c) {
-  return a.W == c.W && a.kind == c.kind && a.merge_warp == c.merge_warp && a.P.tile_cap == c.P.tile_cap &&
+  return a.W == c.W && a.kind == c.kind && a.merge_warp == c.merge_warp && a.P.hash_merge == c.P.hash_merge &&
+         a.P.tile_cap == c.P.tile_cap &&
          a.P.seg_max == c.P.seg_max && a.P.warp_cap == c.P.warp_cap && a.merge_smem_bytes == c.merge_smem_bytes &&
          a.attempt_grid == c.attempt_grid && a.merge_grid == c.merge_grid && a.merge_warp_grid == c.merge_warp_grid;
 }

@@ -787,14 +787,18 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
                      : llrint(q.initiator_threshold * 4294967296.0);
     P.seed = q.seed;
     P.replica = q.replica;
-    P.cap = q.state_capacity > 0 ? q.state_capacity : (int64_t)1 << 20;
+    P.max_det = q.state_capacity > 0 ? q.state_capacity : (int64_t)1 << 20;
+    P.cap = (P.max_det + 3) & ~int64_t(3);
     P.scap = q.spawn_capacity > 0 ? q.spawn_capacity : (int64_t)1 << 21;
     if (P.scap >= ((int64_t)1 << 31)) throw Fail{HANDE_ERR_INVALID, "spawn_capacity must be below 2^31"};
     P.rec_cap = q.record_capacity > 0 ? q.record_capacity : 1 << 16;
     // on-chip tile: distinct new keys (TC, a power of two for the bitonic sort) and
     // main-list entries (SM) per bucket
     if (q.annihilation < 0 || q.annihilation > 2) throw Fail{HANDE_ERR_INVALID, "annihilation must be 0, 1 or 2"};
-    E.merge_warp = q.annihilation != 1;
+    // default: the flat hash path (32-bit list positions and spawn indices),
+    // one warp per bucket for a list that does not fit those
+    P.hash_merge = q.annihilation == 0 && P.cap < ((int64_t)1 << 31) ? 1 : 0;
+    E.merge_warp = !P.hash_merge && q.annihilation != 1;
     // block tiles: sized so that four 256-thread CTAs share an SM for 64- and
     // 128-bit keys (two for 512-bit keys).  Warp path (three 8-warp CTAs per SM,
     // two for 512-bit keys): 128 staged new keys per warp and segments of
@@ -909,10 +913,31 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     P.s_meta = dalloc<uint64_t>(E, scap);
     P.b_key = dalloc<uint64_t>(E, (size_t)scap * E.W);
     P.b_amt = dalloc<int64_t>(E, scap);
-    P.b_flag = dalloc<uint8_t>(E, scap);
-    P.bcount = dalloc<uint32_t>(E, cap);
-    P.boff = dalloc<uint32_t>(E, cap);
-    P.tile_state = dalloc<unsigned long long>(E, cap);
+    if (P.hash_merge) {
+      const int64_t tiles = list_tiles(cap);
+      P.hash_size = 1024;
+      while (P.hash_size < 2 * (uint64_t)scap && P.hash_size < (1ull << 31)) P.hash_size <<= 1;
+      P.hash_tab = dalloc<uint32_t>(E, P.hash_size);
+      CK(cudaMemsetAsync(P.hash_tab, 0, P.hash_size * sizeof(uint32_t), E.stream));
+      P.u_spawn = dalloc<uint32_t>(E, scap);
+      P.u_rank = dalloc<uint32_t>(E, scap);
+      P.n_pos = dalloc<uint32_t>(E, scap);
+      P.n_order = dalloc<uint32_t>(E, scap);
+      P.g_new = dalloc<uint32_t>(E, tiles * kGroups);
+      P.g_keep = dalloc<uint64_t>(E, tiles * kGroups);
+      P.g_pre = dalloc<uint32_t>(E, tiles * kGroups);
+      P.t_keep = dalloc<uint32_t>(E, tiles);
+      P.t_base = dalloc<unsigned long long>(E, tiles);
+      P.occ_draw = dalloc<uint32_t>(E, cap);
+      for (int l = 1; l < kEndLevels && (cap >> (2 * l)) > 0; ++l)
+        P.s_end[l] = dalloc<uint64_t>(E, (size_t)end_stride(cap, l) * E.W);
+    } else {
+      P.b_flag = dalloc<uint8_t>(E, scap);
+      P.bcount = dalloc<uint32_t>(E, cap);
+      P.boff = dalloc<uint32_t>(E, cap);
+      P.tile_state = dalloc<unsigned long long>(E, cap);
+      P.split_key = dalloc<uint64_t>(E, (size_t)cap * E.W);
+    }
     if (E.merge_warp) {
       P.tile_inc = dalloc<unsigned long long>(E, cap);
       P.mcap = cap + scap;   // >= main entries + spawns of one iteration
@@ -921,7 +946,6 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       P.m_hd = dalloc<double>(E, P.mcap);
       P.m_flg = dalloc<uint8_t>(E, P.mcap);
     }
-    P.split_key = dalloc<uint64_t>(E, (size_t)cap * E.W);
     P.st = dalloc<DevState>(E, 1);
     E.check_word = dalloc<unsigned>(E, 4);
     P.rec = dalloc<Record>(E, P.rec_cap);
@@ -1147,7 +1171,7 @@ hande_status hande_set_walkers(hande_ctx* ctx, const uint64_t* keys, const int64
   if (E.failed) return HANDE_ERR_STATE;
   return run_guarded(&E, [&]() -> hande_status {
     const int W = E.W;
-    if (n > E.P.cap) throw Fail{HANDE_ERR_CAPACITY, "more walkers than state_capacity"};
+    if (n > E.P.max_det) throw Fail{HANDE_ERR_CAPACITY, "more walkers than state_capacity"};
     // the keys go to the other list buffer (free between iterations), are
     // checked there and transposed into the list's layout
     const int cur = E.cur;
@@ -1470,15 +1494,17 @@ hande_status hande_diagnostics(hande_ctx* ctx, hande_diag* out) {
     out->bucket_main = hs.sb;
     out->tile_capacity = E.P.tile_cap;
     out->ncore = E.P.ncore;
-    // det pass, attempt scan (2), split, attempts, bucket scan, scatter,
-    // annihilation (1, or 5 on the warp path), new diagonals, finalize, and the
-    // deterministic-space projection (3) once it is active
-    out->launches_per_iteration = 10 + (E.merge_warp ? 4 : 0) + (E.core_active && E.P.ncore > 0 ? 3 : 0);
+    // det pass, attempt scan (2), attempts, then match, decide, place, write; or
+    // split, buckets, bucket scan, scatter, annihilation (1, or 5 on the warp
+    // path), new diagonals, finalize; and the deterministic-space projection (3)
+    // once it is active
+    out->launches_per_iteration = (E.P.hash_merge ? 8 : 11 + (E.merge_warp ? 4 : 0)) +
+                                  (E.core_active && E.P.ncore > 0 ? 3 : 0);
     out->deferred_buckets = hs.ndefer + hs.nbig;
     int64_t nb = std::min<int64_t>(hs.nbuckets, E.P.cap);
     if (nb > 0) {
       std::vector<uint32_t> cnt((size_t)nb);
-      CK(cudaMemcpyAsync(cnt.data(), E.P.bcount, nb * 4, cudaMemcpyDeviceToHost, E.stream));
+      CK(cudaMemcpyAsync(cnt.data(), E.P.hash_merge ? E.P.g_new : E.P.bcount, nb * 4, cudaMemcpyDeviceToHost, E.stream));
       CK(cudaStreamSynchronize(E.stream));
       for (uint32_t c : cnt) out->max_bucket_spawns = std::max<int64_t>(out->max_bucket_spawns, c);
     }

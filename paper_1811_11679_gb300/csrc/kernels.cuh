@@ -5,10 +5,12 @@
 //   det_pass      per determinant: projected-energy terms (App. A.1), initiator
 //                 flag (Sec. 2.1), spawning-attempt count, death/cloning
 //   scan          exclusive scan of attempt counts (attempt space)
-//   split         bucket geometry + splitter keys taken from the sorted main list
 //   core_*        semi-stochastic exact projection inside the deterministic space
-//   attempt       per attempt: Philox draw, excitation, H_ij, spawn amount, bucket id
-//   scan          exclusive scan of bucket counts
+//   attempt       per attempt: Philox draw, excitation, H_ij, spawn amount
+//   match, decide, place, write   the default annihilation (merge_hash.cuh)
+// and with the bucket annihilation (qmc.annihilation = 1 or 2):
+//   split         bucket geometry + splitter keys taken from the sorted main list
+//   bucket, scan  bucket of every spawn, exclusive scan of bucket counts
 //   scatter       spawns -> bucket-contiguous layout (one read + one write)
 //   merge         per bucket: on-chip sort + reduce of its spawns, merge with the
 //                 bucket's main-list segment, initiator rule, real-weight rounding,
@@ -20,6 +22,7 @@
 namespace hande {
 
 constexpr int kMaxW = 8;
+constexpr int kEndLevels = 13;        // block-end levels 1 .. 12 (lists below 2^31 entries)
 constexpr int kScanBlocks = 608;      // 4 x 152 SMs
 constexpr int kScanThreads = 256;
 
@@ -62,6 +65,7 @@ struct DevState {
   unsigned big_ticket;     // block-kernel tickets over all buckets (large-bucket pass)
   int64_t nbig;            // large buckets taken by block tiles
   int64_t ndefer;          // buckets the warp annihilation left to the block kernel
+  unsigned done_ticket;    // blocks of the running kernel that finished (hash annihilation)
   unsigned long long rmax_bits;   // time-step search: largest |H| / p_gen so far (bits of a double >= 0)
 };
 
@@ -75,7 +79,8 @@ struct Params {
   uint64_t seed, replica;
   uint64_t d0[kMaxW];
   // capacities
-  int64_t cap, scap;
+  int64_t cap, scap;     // array strides (cap: a multiple of 4)
+  int64_t max_det;       // most determinants in the list (<= cap)
   int tile_cap, seg_max, rec_cap;
   int bucket_spawns;   // expected spawns per annihilation bucket (sizes the buckets)
   int bucket_new;      // expected distinct new keys per bucket (0 = not used)
@@ -109,6 +114,29 @@ struct Params {
   uint8_t* m_flg;
   int64_t mcap;
   uint64_t* split_key;
+  // hash annihilation (merge_hash.cuh): slots holding a spawn index + 1 (all 0
+  // between iterations); the spawns that represent a new key and their rank of
+  // arrival in their group; survivors by group (keys and amounts in b_key and
+  // b_amt): position in the main list, sorted runs of large groups;
+  // per 64-entry group: survivors, keep bits, entries kept before it in its tile;
+  // per 1024-entry tile: entries kept, {entries, survivors} before it
+  int hash_merge;
+  uint64_t hash_size;
+  uint32_t* hash_tab;
+  uint32_t* u_spawn;
+  uint32_t* u_rank;
+  uint32_t* n_pos;
+  uint32_t* n_order;
+  uint32_t* g_new;
+  uint64_t* g_keep;
+  uint32_t* g_pre;
+  uint32_t* t_keep;
+  unsigned long long* t_base;
+  // of the current list, written by the det pass: each determinant's occupation
+  // draw (top half of Philox word z) and the last keys of its blocks of 4^l
+  // entries (s_end[l], word stride end_stride)
+  uint32_t* occ_draw;
+  uint64_t* s_end[kEndLevels];
   // deterministic space
   int ncore;
   const uint64_t* core_key;
@@ -132,6 +160,10 @@ struct Params {
   Record* rec;
   SysDev sys;
 };
+
+// word stride of the block ends of level l of a list of cap entries (whole
+// nodes of four, so that every node is one aligned sector)
+__host__ __device__ __forceinline__ int64_t end_stride(int64_t cap, int l) { return ((cap >> (2 * l)) + 7) & ~int64_t(3); }
 
 // The block index and grid size a kernel body partitions its work by: the
 // launch's own for a single run and for per-replica grids, a replica's share
@@ -341,6 +373,17 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
   int64_t* pop = P.pop[cur];
   const double* hd = P.hdiag[cur];
   uint8_t* fl = P.flags[cur];
+  if (P.hash_merge) {   // counters of this iteration's spawning and annihilation
+    const int64_t groups = (n / 1024 + 1) * 16;
+    for (int64_t g = vg.b * (int64_t)blockDim.x + threadIdx.x; g < groups; g += (int64_t)vg.n * blockDim.x)
+      P.g_new[g] = 0u;
+    if (vg.b == 0 && threadIdx.x == 0) {
+      st->nbuckets = n / 64 + 1;
+      st->sb = 64;
+      st->nspawn = 0;
+      st->nuniq = 0;
+    }
+  }
   int64_t nw = 0, attsum = 0;
   I128 num{0, 0};
   for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
@@ -360,8 +403,14 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
     bool init = !P.initiator || mag > P.init_thr || is0 || core;
     int64_t na = 0;
     int64_t np = p;
+    Words4 w{};
+    if (p != 0 || (P.hash_merge && P.real_amp)) w = draw<W>(P.seed, P.replica, t, kDetDraw, k);
+    if (P.hash_merge) {
+      P.occ_draw[i] = (uint32_t)(w.z >> 32);
+      for (int l = 1; ((i + 1) & ((int64_t(1) << (2 * l)) - 1)) == 0 && l < kEndLevels; ++l)
+        store_key<W>(P.s_end[l], end_stride(P.cap, l), i >> (2 * l), k);
+    }
     if (p != 0) {
-      Words4 w = draw<W>(P.seed, P.replica, t, kDetDraw, k);
       na = (int64_t)((uint64_t)mag >> 32);
       if (P.real_amp && (w.x >> 32) < ((uint64_t)mag & 0xffffffffull)) na += 1;
       if (!core) {
@@ -583,7 +632,7 @@ static __global__ void __launch_bounds__(1024) kb_scan_buckets(const Params* PP)
 static __global__ void __launch_bounds__(1024) kb_scan_kept(const Params* PP, int cur) {
   const Params& P = PP[blockIdx.y];
   d_scan_one<unsigned long long, unsigned long long>(P.tile_state, P.tile_inc, &P.st->nbuckets,
-                                                     &P.st->ndet[cur ^ 1], P.cap, P.st, &P.st->nnew);
+                                                     &P.st->ndet[cur ^ 1], P.max_det, P.st, &P.st->nnew);
 }
 
 // ------------------------------------------------------------------ buckets
@@ -777,10 +826,6 @@ constexpr int kAttemptThreads = 512;
 constexpr int kAttemptWarps = kAttemptThreads / 32;
 constexpr int kQueue = 64;   // per-warp queue capacity (holds 31 + 32 entries)
 
-template <int W, int SYS>
-__host__ __device__ constexpr int attempt_split_smem() {
-  return W == 8 ? (SYS == SYS_MOLECULE ? 128 : 256) : (W == 2 ? 2048 : 4096);
-}
 // molecular generator tables copied to shared memory for 64-bit keys (at most
 // 64 spin orbitals): the pair records (int4) and the pair unranking table
 constexpr int kStagePairs = 64 * 63 / 2;
@@ -796,8 +841,7 @@ __host__ __device__ constexpr size_t attempt_queue_entry() {
 }
 template <int W, int SYS>
 __host__ __device__ inline size_t attempt_smem_bytes() {
-  return (size_t)attempt_split_smem<W, SYS>() * 8 * W + attempt_stage_bytes<W, SYS>() +
-         (size_t)kAttemptWarps * kQueue * attempt_queue_entry<W, SYS>() + 256;
+  return attempt_stage_bytes<W, SYS>() + (size_t)kAttemptWarps * kQueue * attempt_queue_entry<W, SYS>() + 256;
 }
 
 struct AttemptQueues {
@@ -840,64 +884,23 @@ __device__ __forceinline__ int64_t spawn_amount(const Params& P, uint64_t famt, 
   return neg ? -(int64_t)q : (int64_t)q;
 }
 
-// Bucket search of the spawning kernel: every r-th splitter (coarse, in shared
-// memory when the kernel stages them) then at most r - 1 splitters in global
-// memory.  bucket(k) = number of splitters s_j (1 <= j < nb) with s_j <= k.
-struct SplitIdx {
-  const uint64_t* coarse;   // coarse[c] = s_{c r}, c < nc
-  int64_t cstride, nc, r;
-  const uint64_t* fine;     // all splitters
-  int64_t fstride, nb;
-};
-
+// the top `take` queued spawns of this warp to the staging arrays (meta: the
+// initiator bit; the annihilation adds the spawn's place)
 template <int W>
-__device__ __forceinline__ uint32_t find_bucket(const SplitIdx& sx, const Key<W>& k) {
-  int64_t lo = 1, hi = sx.nc;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (key_le<W>(load_key<W>(sx.coarse, sx.cstride, mid), k)) lo = mid + 1;
-    else hi = mid;
-  }
-  const int64_t c = lo - 1;   // s_{c r} <= k < s_{(c+1) r}
-  int64_t blo = c * sx.r + 1, bhi = c * sx.r + sx.r < sx.nb ? c * sx.r + sx.r : sx.nb;
-  while (blo < bhi) {
-    const int64_t mid = (blo + bhi) >> 1;
-    if (key_le<W>(load_key<W>(sx.fine, sx.fstride, mid), k)) blo = mid + 1;
-    else bhi = mid;
-  }
-  return (uint32_t)(blo - 1);
-}
-
-// the top `take` queued spawns of this warp: bucket, rank, staging slot
-template <int W>
-__device__ void flush_spawns(const Params& P, const AttemptQueues& Q, int& pq_n, int take, const SplitIdx& sx) {
+__device__ void flush_spawns(const Params& P, const AttemptQueues& Q, int& pq_n, int take) {
   DevState* st = P.st;
   const int lane = (int)warp_lane();
-  const bool have = lane < take;
-  Key<W> child;
-  int64_t amt = 0;
-  uint8_t initf = 0;
-  uint32_t bkt = 0;
-  if (have) {
-    const int e = pq_n - take + lane;
-#pragma unroll
-    for (int j = 0; j < W; ++j) child.w[j] = Q.pq_key[j * kQueue + e];
-    amt = Q.pq_amt[e];
-    initf = Q.pq_flg[e];
-    bkt = find_bucket<W>(sx, child);
-  }
-  const unsigned want = __ballot_sync(0xffffffffu, have);
   int64_t base = 0;
-  if (want && lane == 0)
-    base = (int64_t)atomicAdd((unsigned long long*)&st->nspawn, (unsigned long long)__popc(want));
+  if (lane == 0) base = (int64_t)atomicAdd((unsigned long long*)&st->nspawn, (unsigned long long)take);
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (have) {
+  if (lane < take) {
+    const int e = pq_n - take + lane;
     const int64_t slot = base + lane;
-    const uint32_t rank = atomicAdd(&P.bcount[bkt], 1u);
     if (slot < P.scap) {
-      store_key<W>(P.s_key, P.scap, slot, child);
-      P.s_amt[slot] = amt;
-      P.s_meta[slot] = ((uint64_t)bkt << 32) | ((uint64_t)rank << 1) | initf;
+#pragma unroll
+      for (int j = 0; j < W; ++j) P.s_key[j * P.scap + slot] = Q.pq_key[j * kQueue + e];
+      P.s_amt[slot] = Q.pq_amt[e];
+      P.s_meta[slot] = Q.pq_flg[e];
     } else {
       set_error(st, ERR_SPAWN_CAPACITY);
     }
@@ -908,7 +911,7 @@ __device__ void flush_spawns(const Params& P, const AttemptQueues& Q, int& pq_n,
 
 template <int W>
 __device__ __forceinline__ void push_spawn(const Params& P, const AttemptQueues& Q, int& pq_n, bool have,
-                                           const Key<W>& child, int64_t amt, uint8_t initf, const SplitIdx& sx) {
+                                           const Key<W>& child, int64_t amt, uint8_t initf) {
   const unsigned m = __ballot_sync(0xffffffffu, have);
   if (have) {
     const int e = pq_n + __popc(m & ((1u << warp_lane()) - 1u));
@@ -919,14 +922,14 @@ __device__ __forceinline__ void push_spawn(const Params& P, const AttemptQueues&
   }
   pq_n += __popc(m);
   __syncwarp();
-  if (pq_n >= 32) flush_spawns<W>(P, Q, pq_n, 32, sx);
+  if (pq_n >= 32) flush_spawns<W>(P, Q, pq_n, 32);
 }
 
 // the top `take` queued molecular singles: orbitals, H_ia, core test, weight,
 // rounding
 template <int W, int SYS>
 __device__ void flush_singles(const Params& P, const AttemptQueues& Q, int& sq_n, int& pq_n, int take,
-                              const uint64_t* key, const uint8_t* fl, const SplitIdx& sx) {
+                              const uint64_t* key, const uint8_t* fl) {
   const int lane = (int)warp_lane();
   bool have = false;
   Key<W> child;
@@ -956,7 +959,7 @@ __device__ void flush_singles(const Params& P, const AttemptQueues& Q, int& sq_n
   sq_n -= take;
   __syncwarp();
   if (P.tau_search) ratio_max(P, rmax);
-  push_spawn<W>(P, Q, pq_n, have, child, amt, initf, sx);
+  push_spawn<W>(P, Q, pq_n, have, child, amt, initf);
 }
 
 // largest i < n with a[i] <= x, given a[known] <= x (a non-decreasing):
@@ -1026,13 +1029,11 @@ template <int W, int SYS>
 __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid vg) {
   DevState* st = P.st;
   if (st->error) return;
-  constexpr int KS = attempt_split_smem<W, SYS>();
   extern __shared__ __align__(16) unsigned char att_smem[];
-  uint64_t* ssplit = reinterpret_cast<uint64_t*>(att_smem);
   const int wid = threadIdx.x >> 5;
   AttemptQueues Q;
   {
-    unsigned char* p = att_smem + (size_t)KS * 8 * W + attempt_stage_bytes<W, SYS>();
+    unsigned char* p = att_smem + attempt_stage_bytes<W, SYS>();
     const size_t per = kQueue;
     Q.pq_key = reinterpret_cast<uint64_t*>(p) + wid * per * W;
     p += kAttemptWarps * per * 8 * W;
@@ -1059,23 +1060,10 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
   const int64_t t = st->iter + 1;
   const uint64_t* key = P.key[cur];
   const uint8_t* fl = P.flags[cur];
-  // every r-th splitter staged in shared memory (all of them when nb <= KS)
-  SplitIdx sx;
-  sx.r = (nb + KS - 1) / KS;
-  sx.nc = (nb + sx.r - 1) / sx.r;
-  sx.fine = P.split_key;
-  sx.fstride = P.cap;
-  sx.nb = nb;
-  sx.coarse = ssplit;
-  sx.cstride = KS;
-  for (int64_t c = threadIdx.x; c < sx.nc; c += blockDim.x) {
-#pragma unroll
-    for (int j = 0; j < W; ++j) ssplit[j * KS + c] = P.split_key[j * P.cap + c * sx.r];
-  }
   GenTabs gt{P.sys.hb_pair, P.sys.pair_ij};
   if (attempt_stage_bytes<W, SYS>() > 0) {
-    int4* sp = reinterpret_cast<int4*>(att_smem + (size_t)KS * 8 * W);
-    uint16_t* sij = reinterpret_cast<uint16_t*>(att_smem + (size_t)KS * 8 * W + (size_t)kStagePairs * 16);
+    int4* sp = reinterpret_cast<int4*>(att_smem);
+    uint16_t* sij = reinterpret_cast<uint16_t*>(att_smem + (size_t)kStagePairs * 16);
     const int npp = P.sys.nspin * (P.sys.nspin - 1) / 2, nij = P.sys.nel * (P.sys.nel - 1) / 2;
     for (int i = threadIdx.x; i < npp; i += blockDim.x) sp[i] = P.sys.hb_pair[i];
     for (int i = threadIdx.x; i < nij; i += blockDim.x) sij[i] = P.sys.pair_ij[i];
@@ -1182,13 +1170,13 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
       __syncwarp();
     }
     if (P.tau_search) ratio_max(P, rmax);
-    push_spawn<W>(P, Q, pq_n, have, child, amt, initf, sx);
+    push_spawn<W>(P, Q, pq_n, have, child, amt, initf);
     if (SYS == SYS_MOLECULE && sq_n >= 32)
-      flush_singles<W, SYS>(P, Q, sq_n, pq_n, 32, key, fl, sx);
+      flush_singles<W, SYS>(P, Q, sq_n, pq_n, 32, key, fl);
   }
   if (SYS == SYS_MOLECULE && sq_n > 0)
-    flush_singles<W, SYS>(P, Q, sq_n, pq_n, sq_n, key, fl, sx);
-  if (pq_n > 0) flush_spawns<W>(P, Q, pq_n, pq_n, sx);
+    flush_singles<W, SYS>(P, Q, sq_n, pq_n, sq_n, key, fl);
+  if (pq_n > 0) flush_spawns<W>(P, Q, pq_n, pq_n);
 }
 template <int W, int SYS>
 __global__ void __launch_bounds__(kAttemptThreads) k_attempt(Params P, int cur) { d_attempt<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
@@ -1201,6 +1189,36 @@ __global__ void __launch_bounds__(kAttemptThreads, 2) kb_attempt(const Params* P
   __shared__ VGrid vg;
   if (!batch_block(PP, off, R, sP, vg)) return;
   d_attempt<W, SYS>(sP, cur, vg);
+}
+
+// bucket of each staged spawn (the last splitter <= its key) and its rank of
+// arrival there
+template <int W>
+__device__ __forceinline__ void d_bucket(const Params& P, const VGrid vg) {
+  DevState* st = P.st;
+  if (st->error) return;
+  const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap, nb = st->nbuckets;
+  for (int64_t s = (int64_t)vg.b * blockDim.x + threadIdx.x; s < ns; s += (int64_t)vg.n * blockDim.x) {
+    const Key<W> k = load_key<W>(P.s_key, P.scap, s);
+    int64_t lo = 1, hi = nb;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (key_le<W>(load_key<W>(P.split_key, P.cap, mid), k)) lo = mid + 1;
+      else hi = mid;
+    }
+    const uint32_t rank = atomicAdd(&P.bcount[lo - 1], 1u);
+    P.s_meta[s] = ((uint64_t)(lo - 1) << 32) | ((uint64_t)rank << 1) | (P.s_meta[s] & 1u);
+  }
+}
+template <int W>
+__global__ void __launch_bounds__(256) k_bucket(Params P) { d_bucket<W>(P, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+// the same for replica blockIdx.y of a batch (parameter blocks PP[replica])
+template <int W>
+__global__ void __launch_bounds__(256) kb_bucket(const Params* PP, const int* off, int R) {
+  __shared__ Params sP;
+  __shared__ VGrid vg;
+  if (!batch_block(PP, off, R, sP, vg)) return;
+  d_bucket<W>(sP, vg);
 }
 
 template <int W>
@@ -1927,7 +1945,7 @@ __device__ __forceinline__ void d_merge(const Params& P, int cur, int staged, co
           if (threadIdx.x == 0) {
             s_base = base;
             s_abort = ab;
-            if (!ab && (int64_t)(base + nkeep) > P.cap) {
+            if (!ab && (int64_t)(base + nkeep) > P.max_det) {
               set_error(st, ERR_STATE_CAPACITY);
               s_abort = 1;
             }
@@ -2053,7 +2071,7 @@ __device__ __forceinline__ void d_merge(const Params& P, int cur, int staged, co
         if (threadIdx.x == 0) {
           s_base = base;
           s_abort = ab;
-          if (!ab && (int64_t)(base + total) > P.cap) {
+          if (!ab && (int64_t)(base + total) > P.max_det) {
             set_error(st, ERR_STATE_CAPACITY);
             s_abort = 1;
           }
@@ -2100,12 +2118,11 @@ __global__ void __launch_bounds__(kMergeThreads, (W == 8 ? 2 : 4)) kb_merge(cons
 }
 
 // ------------------------------------------------------------------ finalize
-__device__ __forceinline__ void d_finalize(const Params& P, int cur) {
+// shift update and record of the iteration (one thread): the new list has ndet
+// entries holding nw walkers
+__device__ __forceinline__ void finalize_iteration(const Params& P, int64_t ndet, int64_t nw) {
   DevState* st = P.st;
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (st->error) return;
   const int64_t t = st->iter + 1;
-  const int64_t nw = st->nw_post;
   if (st->vary) {
     if (t % P.period == 0) {
       double ratio = __ddiv_rn((double)nw, (double)st->nw_ref);
@@ -2123,7 +2140,7 @@ __device__ __forceinline__ void d_finalize(const Params& P, int cur) {
   r.nw_pre = st->nw_pre;
   r.n0 = st->n0;
   r.nw_post = nw;
-  r.ndet = st->ndet[cur ^ 1];
+  r.ndet = ndet;
   r.natt = st->natt;
   r.nspawn = st->nspawn;
   r.tau = P.tau;
@@ -2140,6 +2157,12 @@ __device__ __forceinline__ void d_finalize(const Params& P, int cur) {
   st->num[0] = 0;
   st->num[1] = 0;
   st->nw_post = 0;
+}
+__device__ __forceinline__ void d_finalize(const Params& P, int cur) {
+  DevState* st = P.st;
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (st->error) return;
+  finalize_iteration(P, st->ndet[cur ^ 1], st->nw_post);
 }
 static __global__ void k_finalize(Params P, int cur) { d_finalize(P, cur); }
 // the same for replica blockIdx.y of a batch (parameter blocks PP[replica])
@@ -2209,4 +2232,5 @@ __global__ void k_eref(Params P) {
 
 }  // namespace hande
 
+#include "merge_hash.cuh"
 #include "merge_warp.cuh"

@@ -127,19 +127,22 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
     // branch beside the det pass and the attempt scan; the core update waits
     // for both (the det pass reads the core populations).  A failing record or
     // wait invalidates the capture, which ending the capture reports.
-    (void)(cudaEventRecord(E.ev_fork, s));
-    (void)(cudaStreamWaitEvent(E.aux_stream, E.ev_fork, 0));
-    k_split<W><<<kScanBlocks, 256, 0, E.aux_stream>>>(P, cur);
+    const bool branch = with_core || !P.hash_merge;
+    if (branch) {
+      (void)(cudaEventRecord(E.ev_fork, s));
+      (void)(cudaStreamWaitEvent(E.aux_stream, E.ev_fork, 0));
+    }
+    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, E.aux_stream>>>(P, cur);
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, E.aux_stream>>>(P, cur);
       k_core_spmv<<<(int)(((int64_t)P.ncore * 32 + 255) / 256), 256, 0, E.aux_stream>>>(P, cur);
     }
-    (void)(cudaEventRecord(E.ev_join, E.aux_stream));
+    if (branch) (void)(cudaEventRecord(E.ev_join, E.aux_stream));
     k_det_pass<W, SYS><<<kScanBlocks, kScanThreads, 0, s>>>(P, cur);
     k_scan_partials_i64<<<1, 1024, 0, s>>>(P.part, kScanBlocks, st_field_i64(st, offsetof(DevState, natt)), st);
     k_scan_apply<int64_t><<<kScanBlocks, kScanThreads, 0, s>>>(
         P.natt, P.att_begin, st_field_i64(st, offsetof(DevState, ndet) + 8 * cur), P.part, st);
-    (void)(cudaStreamWaitEvent(s, E.ev_join, 0));
+    if (branch) (void)(cudaStreamWaitEvent(s, E.ev_join, 0));
     if (with_core) k_core_apply<<<ncb, 256, 0, s>>>(P, cur);
   } else {
     mark(0);
@@ -149,7 +152,7 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
     k_scan_apply<int64_t><<<kScanBlocks, kScanThreads, 0, s>>>(
         P.natt, P.att_begin, st_field_i64(st, offsetof(DevState, ndet) + 8 * cur), P.part, st);
     mark(2);
-    k_split<W><<<kScanBlocks, 256, 0, s>>>(P, cur);
+    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, s>>>(P, cur);
     mark(3);
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, s>>>(P, cur);
@@ -160,6 +163,19 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
   mark(4);
   k_attempt<W, SYS><<<E.attempt_grid, kAttemptThreads, attempt_smem_bytes<W, SYS>(), s>>>(P, cur);
   mark(5);
+  if (P.hash_merge) {
+    mark(6);
+    mark(7);
+    k_match<W><<<E.attempt_grid * 2, kMatchThreads, 0, s>>>(P, cur);
+    k_decide<W><<<E.attempt_grid * 2, kListThreads, 0, s>>>(P, cur);
+    k_place<W><<<E.attempt_grid, 256, 0, s>>>(P, cur);
+    k_write<W, SYS><<<E.attempt_grid * 2, kListThreads, 0, s>>>(P, cur);
+    mark(8);
+    mark(9);
+    mark(10);
+    return;
+  }
+  k_bucket<W><<<E.attempt_grid * 4, 256, 0, s>>>(P);
   int64_t* nbk = st_field_i64(st, offsetof(DevState, nbuckets));
   k_scan_one<uint32_t, uint32_t><<<1, 1024, 0, s>>>(P.bcount, P.boff, nbk,
                                                     st_field_i64(st, offsetof(DevState, scan_total)), -1, st);
@@ -181,7 +197,7 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
       k_merge<W, SYS><<<E.merge_grid, kMergeThreads, E.merge_smem_bytes, s>>>(P, cur, 1);
     }
     k_scan_one<unsigned long long, unsigned long long><<<1, 1024, 0, s>>>(
-        P.tile_state, P.tile_inc, nbk, st_field_i64(st, offsetof(DevState, ndet) + 8 * (cur ^ 1)), P.cap, st,
+        P.tile_state, P.tile_inc, nbk, st_field_i64(st, offsetof(DevState, ndet) + 8 * (cur ^ 1)), P.max_det, st,
         st_field_i64(st, offsetof(DevState, nnew)));
     k_merge_copy<W><<<E.attempt_grid * 2, 256, 0, s>>>(P, cur);
   } else {
@@ -211,20 +227,31 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
   auto off = [&](int p) { return G.d_off + (size_t)p * (R + 1); };
   auto blocks = [&](int p) { return (unsigned)(G.plan.budget[p] + R); };
   kb_plan<<<1, 32, 0, s>>>(PP, R, cur, G.plan, G.d_off);
-  (void)cudaEventRecord(fork, s);
-  (void)cudaStreamWaitEvent(aux, fork, 0);
-  kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
+  const bool hash = E0.P.hash_merge != 0, branch = !hash || G.max_ncore > 0;
+  if (branch) {
+    (void)cudaEventRecord(fork, s);
+    (void)cudaStreamWaitEvent(aux, fork, 0);
+  }
+  if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
   if (G.max_ncore > 0) {
     kb_core_locate<W><<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
     kb_core_spmv<<<dim3((unsigned)(((int64_t)G.max_ncore * 32 + 255) / 256), R), 256, 0, aux>>>(PP, cur);
   }
-  (void)cudaEventRecord(join, aux);
+  if (branch) (void)cudaEventRecord(join, aux);
   kb_det_pass<W, SYS><<<blocks(0), kScanThreads, 0, s>>>(PP, off(0), R, cur);
   kb_scan_natt<<<dim3(1, R), 1024, 0, s>>>(PP, off(0), R);
   kb_scan_att<<<blocks(0), kScanThreads, 0, s>>>(PP, off(0), R, cur);
-  (void)cudaStreamWaitEvent(s, join, 0);
+  if (branch) (void)cudaStreamWaitEvent(s, join, 0);
   if (G.max_ncore > 0) kb_core_apply<<<dim3(ncb, R), 256, 0, s>>>(PP, cur);
   kb_attempt<W, SYS><<<blocks(1), kAttemptThreads, attempt_smem_bytes<W, SYS>(), s>>>(PP, off(1), R, cur);
+  if (hash) {
+    kb_match<W><<<blocks(2), kMatchThreads, 0, s>>>(PP, off(2), R, cur);
+    kb_decide<W><<<blocks(5), kListThreads, 0, s>>>(PP, off(5), R, cur);
+    kb_place<W><<<blocks(6), 256, 0, s>>>(PP, off(6), R, cur);
+    kb_write<W, SYS><<<blocks(5), kListThreads, 0, s>>>(PP, off(5), R, cur);
+    return;
+  }
+  kb_bucket<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
   kb_scan_buckets<<<dim3(1, R), 1024, 0, s>>>(PP);
   kb_scatter<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
   if (E0.merge_warp) {
