@@ -908,6 +908,8 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     P.natt = dalloc<int64_t>(E, cap);
     P.att_begin = dalloc<int64_t>(E, cap);
     P.part = dalloc<int64_t>(E, kScanBlocks + 1);
+    P.det_state = dalloc<unsigned long long>(E, cap / kDetTile + 2);
+    CK(cudaMemsetAsync(P.det_state, 0, (cap / kDetTile + 2) * sizeof(unsigned long long), E.stream));
     P.s_key = dalloc<uint64_t>(E, (size_t)scap * E.W);
     P.s_amt = dalloc<int64_t>(E, scap);
     P.s_meta = dalloc<uint64_t>(E, scap);
@@ -923,7 +925,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       P.u_rank = dalloc<uint32_t>(E, scap);
       P.n_pos = dalloc<uint32_t>(E, scap);
       P.n_order = dalloc<uint32_t>(E, scap);
-      P.g_new = dalloc<uint32_t>(E, tiles * kGroups);
+      P.g_new = dalloc<uint32_t>(E, (tiles + 1) * kGroups);   // the det pass clears one tile ahead
       P.g_keep = dalloc<uint64_t>(E, tiles * kGroups);
       P.g_pre = dalloc<uint32_t>(E, tiles * kGroups);
       P.t_keep = dalloc<uint32_t>(E, tiles);
@@ -1494,11 +1496,10 @@ hande_status hande_diagnostics(hande_ctx* ctx, hande_diag* out) {
     out->bucket_main = hs.sb;
     out->tile_capacity = E.P.tile_cap;
     out->ncore = E.P.ncore;
-    // det pass, attempt scan (2), attempts, then match, decide, place, write; or
-    // split, buckets, bucket scan, scatter, annihilation (1, or 5 on the warp
+    // det pass, attempts, then match, decide, place, write; or split, buckets, bucket scan, scatter, annihilation (1, or 5 on the warp
     // path), new diagonals, finalize; and the deterministic-space projection (3)
     // once it is active
-    out->launches_per_iteration = (E.P.hash_merge ? 8 : 11 + (E.merge_warp ? 4 : 0)) +
+    out->launches_per_iteration = (E.P.hash_merge ? 6 : 9 + (E.merge_warp ? 4 : 0)) +
                                   (E.core_active && E.P.ncore > 0 ? 3 : 0);
     out->deferred_buckets = hs.ndefer + hs.nbig;
     int64_t nb = std::min<int64_t>(hs.nbuckets, E.P.cap);

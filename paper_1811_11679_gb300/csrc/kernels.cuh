@@ -65,6 +65,7 @@ struct DevState {
   unsigned big_ticket;     // block-kernel tickets over all buckets (large-bucket pass)
   int64_t nbig;            // large buckets taken by block tiles
   int64_t ndefer;          // buckets the warp annihilation left to the block kernel
+  unsigned det_ticket;     // tiles of the det pass
   unsigned done_ticket;    // blocks of the running kernel that finished (hash annihilation)
   unsigned long long rmax_bits;   // time-step search: largest |H| / p_gen so far (bits of a double >= 0)
 };
@@ -94,6 +95,7 @@ struct Params {
   int64_t* natt;
   int64_t* att_begin;
   int64_t* part;         // scan partials, kScanBlocks + 1
+  unsigned long long* det_state;   // look-back states of the det pass's tiles (0 between iterations)
   // spawns
   uint64_t* s_key;
   int64_t* s_amt;
@@ -357,95 +359,227 @@ __device__ __forceinline__ void block_chunk(int64_t n, int64_t& beg, int64_t& en
 }
 
 // ------------------------------------------------------------------ det pass
+// Decoupled look-back (single-pass chained scan) over the tiles' counts in
+// state[] (all 0 before the kernel), run by one warp: each step reads 32
+// predecessor states at once.  Tiles are
+// taken in ticket order, so every predecessor is owned by a running CTA and
+// publishes its count without waiting: the spin always ends, and is bounded
+// anyway.  Returns the exclusive prefix (all lanes); sets *abort on failure.
+__device__ __forceinline__ unsigned long long lookback_warp(DevState* st, unsigned long long* state, int64_t b,
+                                                            unsigned long long count, int* abort) {
+  const unsigned long long AGG = 1ull << 62, INC = 2ull << 62, MASK = (1ull << 62) - 1;
+  const int lane = (int)warp_lane();
+  if (b == 0) {
+    if (lane == 0) atomicExch(&state[0], INC | count);
+    return 0;
+  }
+  if (lane == 0) atomicExch(&state[b], AGG | count);
+  unsigned long long excl = 0;
+  int64_t p = b - 1;
+  long long spins = 0;
+  for (;;) {
+    const int64_t idx = p - lane;
+    const unsigned long long v = idx >= 0 ? *(volatile const unsigned long long*)&state[idx] : INC;
+    const unsigned long long s = v >> 62;
+    const unsigned inc = __ballot_sync(0xffffffffu, s == 2);
+    const unsigned none = __ballot_sync(0xffffffffu, s == 0);
+    const int first = inc ? __ffs(inc) - 1 : 31;
+    const unsigned need = first == 31 ? 0xffffffffu : ((2u << first) - 1u);
+    if (none & need) {   // a state we need is not published yet
+      ++spins;
+      __nanosleep(64);
+      if ((spins & 255) == 0 && *(volatile unsigned*)&st->error) {
+        *abort = 1;   // another tile failed: give up without adding an error
+        return 0;
+      }
+      if (spins > (1ll << 20)) {
+        if (lane == 0) set_error(st, ERR_TIMEOUT);
+        *abort = 1;
+        return 0;
+      }
+      continue;
+    }
+    unsigned long long add = (lane <= first) ? (v & MASK) : 0ull;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
+    excl += add;
+    if (inc) break;
+    p -= 32;
+  }
+  if (lane == 0) atomicExch(&state[b], INC | (excl + count));
+  return excl;
+}
+
+// One pass over the list: estimators, initiator flags, death, attempt counts and
+// their exclusive scan (att_begin), in tiles of 1024 entries taken in ticket
+// order.  The scan is chained through the tiles (look-back) instead of a second
+// and third kernel over the counts: those cost 21 us of a 930 us iteration on
+// 2.3e6 determinants, and two launches of the 17 of a small one.  Entries
+// connected to the reference (a percent of a large list) are queued and their
+// matrix elements evaluated by full warps while warp 0 looks back.
+// Bound: the FP64 unit (death: five operations per entry) and Philox issue.
+constexpr int kDetThreads = 512;
+constexpr int kDetItems = 2;
+constexpr int kDetTile = kDetThreads * kDetItems;   // 1024
+constexpr int kDetWarps = kDetThreads / 32;
+static_assert(kDetItems * kDetWarps == 32, "one warp scans the tile's warp sums");
+
 template <int W, int SYS>
 __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid vg) {
   DevState* st = P.st;
-  if (st->error) return;
   __shared__ int64_t sh64[32];
   __shared__ I128 sh128[32];
+  __shared__ unsigned long long wpre[32];
+  __shared__ uint16_t queue[kDetTile];   // entries connected to the reference
+  __shared__ int64_t queue_n[kDetTile];  // and their populations before death
+  __shared__ int s_qn, s_abort;
+  __shared__ unsigned s_tile;
+  if (__syncthreads_or((int)st->error)) return;
   const int64_t n = st->ndet[cur];
   const int64_t t = st->iter + 1;
   const double S = st->shift;
   const Key<W> d0 = ref_key<W>(P);
-  int64_t beg, end;
-  block_chunk(n, beg, end, vg);
-  uint64_t* key = P.key[cur];
+  const uint64_t* key = P.key[cur];
   int64_t* pop = P.pop[cur];
   const double* hd = P.hdiag[cur];
   uint8_t* fl = P.flags[cur];
-  if (P.hash_merge) {   // counters of this iteration's spawning and annihilation
-    const int64_t groups = (n / 1024 + 1) * 16;
-    for (int64_t g = vg.b * (int64_t)blockDim.x + threadIdx.x; g < groups; g += (int64_t)vg.n * blockDim.x)
-      P.g_new[g] = 0u;
-    if (vg.b == 0 && threadIdx.x == 0) {
-      st->nbuckets = n / 64 + 1;
-      st->sb = 64;
-      st->nspawn = 0;
-      st->nuniq = 0;
-    }
+  const int lane = (int)warp_lane(), wid = (int)(threadIdx.x >> 5);
+  const int64_t tiles = (n + kDetTile - 1) / kDetTile;
+  if (vg.b == 0 && threadIdx.x == 0 && P.hash_merge) {   // counters of the spawning and the annihilation
+    st->nbuckets = n / 64 + 1;
+    st->sb = 64;
+    st->nspawn = 0;
+    st->nuniq = 0;
   }
-  int64_t nw = 0, attsum = 0;
+  int64_t nw = 0;
   I128 num{0, 0};
-  for (int64_t i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    Key<W> k = load_key<W>(key, P.cap, i);
-    int64_t p = pop[i];
-    uint8_t f = fl[i] & F_CORE;
-    bool core = f != 0;
-    bool is0 = key_eq<W>(k, d0);
-    int64_t mag = iabs64(p);
-    nw += mag;
-    if (is0) {
-      st->n0 = p;
-    } else if (p != 0 && key_popc_xor<W>(k, d0) <= 4) {
-      double h0j = h_elem<W, SYS>(P.sys, k, d0);
-      i128_add(num, fixed_term(p, h0j));
+  for (;;) {
+    if (threadIdx.x == 0) {
+      s_tile = atomicAdd(&st->det_ticket, 1u);
+      s_qn = 0;
+      s_abort = 0;
     }
-    bool init = !P.initiator || mag > P.init_thr || is0 || core;
-    int64_t na = 0;
-    int64_t np = p;
-    Words4 w{};
-    if (p != 0 || (P.hash_merge && P.real_amp)) w = draw<W>(P.seed, P.replica, t, kDetDraw, k);
-    if (P.hash_merge) {
-      P.occ_draw[i] = (uint32_t)(w.z >> 32);
-      for (int l = 1; ((i + 1) & ((int64_t(1) << (2 * l)) - 1)) == 0 && l < kEndLevels; ++l)
-        store_key<W>(P.s_end[l], end_stride(P.cap, l), i >> (2 * l), k);
-    }
-    if (p != 0) {
-      na = (int64_t)((uint64_t)mag >> 32);
-      if (P.real_amp && (w.x >> 32) < ((uint64_t)mag & 0xffffffffull)) na += 1;
-      if (!core) {
-        double d = __dmul_rn(P.tau, __dsub_rn(__ldg(&hd[i]), S));
-        if (P.real_amp) {
-          np = p - __double2ll_rn(__dmul_rn(d, (double)p));
-        } else {
-          int64_t nwk = mag >> 32;
-          double x = __dmul_rn(fabs(d), (double)nwk);
-          double flo = floor(x);
-          int64_t kk = (int64_t)flo;
-          if (draw_unit(w.y) < __dsub_rn(x, flo)) kk += 1;
-          int64_t nn = d > 0.0 ? nwk - kk : nwk + kk;
-          np = (p < 0 ? -nn : nn) * kOne;
-        }
-        if (iabs64(np) >= (int64_t(1) << 62)) set_error(st, ERR_OVERFLOW);
-        if (np != p) pop[i] = np;
+    __syncthreads();
+    const int64_t tile = s_tile, base = tile * kDetTile;
+    if (tile >= tiles) break;
+    if (P.hash_merge && threadIdx.x < 32) P.g_new[tile * 16 + threadIdx.x] = 0u;   // and the groups behind the list
+    unsigned long long na[kDetItems], pre[kDetItems];
+    // all loads of the thread's entries before the first use
+    Key<W> kk[kDetItems];
+    int64_t pp[kDetItems];
+    double hh[kDetItems];
+    uint8_t ff[kDetItems];
+#pragma unroll
+    for (int u = 0; u < kDetItems; ++u) {
+      const int64_t i = base + u * kDetThreads + threadIdx.x;
+      if (i < n) {
+        kk[u] = load_key<W>(key, P.cap, i);
+        pp[u] = pop[i];
+        ff[u] = fl[i];
+        hh[u] = __ldg(&hd[i]);
       }
     }
-    fl[i] = f | (init ? F_INIT : 0) | (p < 0 ? F_NEG : 0) | (is0 ? F_REF : 0);
-    P.natt[i] = na;
-    attsum += na;
+#pragma unroll
+    for (int u = 0; u < kDetItems; ++u) {
+      const int64_t i = base + u * kDetThreads + threadIdx.x;
+      na[u] = 0;
+      if (i < n) {
+        const Key<W>& k = kk[u];
+        const int64_t p = pp[u];
+        const uint8_t f = ff[u] & F_CORE;
+        const bool core = f != 0;
+        const bool is0 = key_eq<W>(k, d0);
+        const int64_t mag = iabs64(p);
+        nw += mag;
+        if (is0) {
+          st->n0 = p;
+        } else if (p != 0 && key_popc_xor<W>(k, d0) <= 4) {
+          const int q = atomicAdd(&s_qn, 1);
+          queue[q] = (uint16_t)(i - base);
+          queue_n[q] = p;
+        }
+        const bool init = !P.initiator || mag > P.init_thr || is0 || core;
+        Words4 w{};
+        if (p != 0 || (P.hash_merge && P.real_amp)) w = draw<W>(P.seed, P.replica, t, kDetDraw, k);
+        if (P.hash_merge) {
+          P.occ_draw[i] = (uint32_t)(w.z >> 32);
+          for (int l = 1; ((i + 1) & ((int64_t(1) << (2 * l)) - 1)) == 0 && l < kEndLevels; ++l)
+            store_key<W>(P.s_end[l], end_stride(P.cap, l), i >> (2 * l), k);
+        }
+        if (p != 0) {
+          na[u] = (uint64_t)mag >> 32;
+          if (P.real_amp && (w.x >> 32) < ((uint64_t)mag & 0xffffffffull)) na[u] += 1;
+          if (!core) {
+            const double d = __dmul_rn(P.tau, __dsub_rn(hh[u], S));
+            int64_t np;
+            if (P.real_amp) {
+              np = p - __double2ll_rn(__dmul_rn(d, (double)p));
+            } else {
+              int64_t nwk = mag >> 32;
+              double x = __dmul_rn(fabs(d), (double)nwk);
+              double flo = floor(x);
+              int64_t kk = (int64_t)flo;
+              if (draw_unit(w.y) < __dsub_rn(x, flo)) kk += 1;
+              int64_t nn = d > 0.0 ? nwk - kk : nwk + kk;
+              np = (p < 0 ? -nn : nn) * kOne;
+            }
+            if (iabs64(np) >= (int64_t(1) << 62)) set_error(st, ERR_OVERFLOW);
+            if (np != p) pop[i] = np;
+          }
+        }
+        fl[i] = f | (init ? F_INIT : 0) | (p < 0 ? F_NEG : 0) | (is0 ? F_REF : 0);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kDetItems; ++u) {
+      unsigned long long x = na[u];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      pre[u] = x - na[u];
+      if (lane == 31) wpre[u * kDetWarps + wid] = x;
+    }
+    __syncthreads();
+    if (wid == 0) {
+      const unsigned long long v = wpre[lane];
+      unsigned long long x = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      const unsigned long long total = __shfl_sync(0xffffffffu, x, 31);
+      int ab = 0;
+      const unsigned long long before = lookback_warp(st, P.det_state, tile, total, &ab);
+      wpre[lane] = before + x - v;
+      if (lane == 0) {
+        if (ab) s_abort = 1;
+        if (tile == tiles - 1) st->natt = (int64_t)(before + total);
+      }
+    } else {
+      for (int q = (int)threadIdx.x - 32; q < s_qn; q += kDetThreads - 32)
+        i128_add(num, fixed_term(queue_n[q], h_connected<W, SYS>(P.sys, load_key<W>(key, P.cap, base + queue[q]), d0)));
+    }
+    __syncthreads();
+    if (s_abort) break;
+#pragma unroll
+    for (int u = 0; u < kDetItems; ++u) {
+      const int64_t i = base + u * kDetThreads + threadIdx.x;
+      if (i < n) P.att_begin[i] = (int64_t)(wpre[u * kDetWarps + wid] + pre[u]);
+    }
   }
-  int64_t a = block_sum<int64_t>(attsum, sh64);
-  if (threadIdx.x == 0) P.part[vg.b] = a;
-  int64_t b = block_sum<int64_t>(nw, sh64);
+  const int64_t b = block_sum<int64_t>(nw, sh64);
   if (threadIdx.x == 0 && b) atomicAdd((unsigned long long*)&st->nw_pre, (unsigned long long)b);
-  I128 c = block_sum_i128(num, sh128);
+  const I128 c = block_sum_i128(num, sh128);
   if (threadIdx.x == 0 && (c.lo | (uint64_t)c.hi)) atomic_add_i128(st->num, c);
 }
 template <int W, int SYS>
-__global__ void __launch_bounds__(kScanThreads) k_det_pass(Params P, int cur) { d_det_pass<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+__global__ void __launch_bounds__(kDetThreads, W == 8 ? 1 : 2) k_det_pass(Params P, int cur) { d_det_pass<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
 // the same for replica blockIdx.y of a batch (parameter blocks PP[replica])
 template <int W, int SYS>
-__global__ void __launch_bounds__(kScanThreads) kb_det_pass(const Params* PP, const int* off, int R, int cur) {
+__global__ void __launch_bounds__(kDetThreads, W == 8 ? 1 : 2) kb_det_pass(const Params* PP, const int* off, int R, int cur) {
   __shared__ Params sP;
   __shared__ VGrid vg;
   if (!batch_block(PP, off, R, sP, vg)) return;
@@ -615,16 +749,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const T* in, const
 }
 
 // batched forms of the scans, pointers taken from replica blockIdx.y's block
-static __global__ void kb_scan_natt(const Params* PP, const int* off, int R) {
-  const Params& P = PP[blockIdx.y];
-  d_scan_partials_i64(P.part, off[blockIdx.y + 1] - off[blockIdx.y], &P.st->natt, P.st);
-}
-static __global__ void __launch_bounds__(kScanThreads) kb_scan_att(const Params* PP, const int* off, int R, int cur) {
-  __shared__ Params sP;
-  __shared__ VGrid vg;
-  if (!batch_block(PP, off, R, sP, vg)) return;
-  d_scan_apply<int64_t>(sP.natt, sP.att_begin, &sP.st->ndet[cur], sP.part, sP.st, vg);
-}
 static __global__ void __launch_bounds__(1024) kb_scan_buckets(const Params* PP) {
   const Params& P = PP[blockIdx.y];
   d_scan_one<uint32_t, uint32_t>(P.bcount, P.boff, &P.st->nbuckets, &P.st->scan_total, -1, P.st, nullptr);
@@ -1056,7 +1180,6 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
   }
   const int64_t natt = st->natt;
   const int64_t n = st->ndet[cur];
-  const int64_t nb = st->nbuckets;
   const int64_t t = st->iter + 1;
   const uint64_t* key = P.key[cur];
   const uint8_t* fl = P.flags[cur];
@@ -1198,6 +1321,10 @@ __device__ __forceinline__ void d_bucket(const Params& P, const VGrid vg) {
   DevState* st = P.st;
   if (st->error) return;
   const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap, nb = st->nbuckets;
+  // the det pass's look-back states, for the next iteration
+  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c * kDetTile < P.cap && c * kDetTile < nb * st->sb;
+       c += (int64_t)vg.n * blockDim.x)
+    P.det_state[c] = 0ull;
   for (int64_t s = (int64_t)vg.b * blockDim.x + threadIdx.x; s < ns; s += (int64_t)vg.n * blockDim.x) {
     const Key<W> k = load_key<W>(P.s_key, P.scap, s);
     int64_t lo = 1, hi = nb;
@@ -1712,56 +1839,6 @@ __device__ int64_t acc_write(const Params& P, MergeSmem<W>& m, const MergeCtx& c
   return nwsum;
 }
 
-// Decoupled look-back (single-pass chained scan) over bucket output counts,
-// run by one warp: each step reads 32 predecessor states at once.  Buckets are
-// taken in ticket order, so every predecessor is owned by a running CTA and
-// publishes its count without waiting: the spin always ends, and is bounded
-// anyway.  Returns the exclusive prefix (all lanes); sets *abort on failure.
-__device__ __forceinline__ unsigned long long lookback_warp(const Params& P, int64_t b, uint32_t count, int* abort) {
-  DevState* st = P.st;
-  const unsigned long long AGG = 1ull << 62, INC = 2ull << 62, MASK = (1ull << 62) - 1;
-  const int lane = (int)warp_lane();
-  if (b == 0) {
-    if (lane == 0) atomicExch(&P.tile_state[0], INC | (unsigned long long)count);
-    return 0;
-  }
-  if (lane == 0) atomicExch(&P.tile_state[b], AGG | (unsigned long long)count);
-  unsigned long long excl = 0;
-  int64_t p = b - 1;
-  long long spins = 0;
-  for (;;) {
-    const int64_t idx = p - lane;
-    const unsigned long long v = idx >= 0 ? *(volatile const unsigned long long*)&P.tile_state[idx] : INC;
-    const unsigned long long s = v >> 62;
-    const unsigned inc = __ballot_sync(0xffffffffu, s == 2);
-    const unsigned none = __ballot_sync(0xffffffffu, s == 0);
-    const int first = inc ? __ffs(inc) - 1 : 31;
-    const unsigned need = first == 31 ? 0xffffffffu : ((2u << first) - 1u);
-    if (none & need) {   // a state we need is not published yet
-      ++spins;
-      __nanosleep(64);
-      if ((spins & 255) == 0 && *(volatile unsigned*)&st->error) {
-        *abort = 1;   // another tile failed: give up without adding an error
-        return 0;
-      }
-      if (spins > (1ll << 20)) {
-        if (lane == 0) set_error(st, ERR_TIMEOUT);
-        *abort = 1;
-        return 0;
-      }
-      continue;
-    }
-    unsigned long long add = (lane <= first) ? (v & MASK) : 0ull;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
-    excl += add;
-    if (inc) break;
-    p -= 32;
-  }
-  if (lane == 0) atomicExch(&P.tile_state[b], INC | (excl + count));
-  return excl;
-}
-
 constexpr int kMergeThreads = 256;
 
 template <int W, int SYS>
@@ -1941,7 +2018,7 @@ __device__ __forceinline__ void d_merge(const Params& P, int cur, int staged, co
         }
         if (threadIdx.x < 32) {
           int ab = 0;
-          const unsigned long long base = lookback_warp(P, b, nkeep, &ab);
+          const unsigned long long base = lookback_warp(st, P.tile_state, b, nkeep, &ab);
           if (threadIdx.x == 0) {
             s_base = base;
             s_abort = ab;
@@ -2067,7 +2144,7 @@ __device__ __forceinline__ void d_merge(const Params& P, int cur, int staged, co
         }
       } else if (threadIdx.x < 32) {
         int ab = 0;
-        const unsigned long long base = lookback_warp(P, b, total, &ab);
+        const unsigned long long base = lookback_warp(st, P.tile_state, b, total, &ab);
         if (threadIdx.x == 0) {
           s_base = base;
           s_abort = ab;
@@ -2152,6 +2229,7 @@ __device__ __forceinline__ void finalize_iteration(const Params& P, int64_t ndet
   r.num = fixed_to_double(num);
   P.rec[(t - 1) % P.rec_cap] = r;
   st->iter = t;
+  st->det_ticket = 0;
   st->nw_pre = 0;
   st->n0 = 0;
   st->num[0] = 0;

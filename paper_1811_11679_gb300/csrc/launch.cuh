@@ -115,54 +115,55 @@ __global__ void k_sel_gather(Params P, int cur, uint64_t* core_key, int64_t ncor
 template <int W, int SYS>
 void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_t* ev) {
   Params& P = E.P;
-  DevState* st = P.st;
+  [[maybe_unused]] DevState* st = P.st;
   auto mark = [&](int k) {
     if (ev) cudaEventRecord(ev[k], s);
   };
   const bool with_core = core && P.ncore > 0;
   const int ncb = (P.ncore + 255) / 256;
-  if (!ev && E.aux_stream) {
-    // captured iteration: the bucket split and the deterministic-space product
-    // (they read only keys, the core populations and the CSR) run on a second
-    // branch beside the det pass and the attempt scan; the core update waits
-    // for both (the det pass reads the core populations).  A failing record or
-    // wait invalidates the capture, which ending the capture reports.
-    const bool branch = with_core || !P.hash_merge;
-    if (branch) {
-      (void)(cudaEventRecord(E.ev_fork, s));
-      (void)(cudaStreamWaitEvent(E.aux_stream, E.ev_fork, 0));
-    }
-    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, E.aux_stream>>>(P, cur);
+  const int spmv_blocks = (int)(((int64_t)P.ncore * 32 + 255) / 256);
+  const bool branch = !ev && E.aux_stream && (with_core || !P.hash_merge);
+  cudaStream_t aux = branch ? E.aux_stream : s;
+  // captured iteration: the bucket split and the deterministic-space product
+  // (they read only keys, the core populations and the CSR) run on a second
+  // branch beside the det pass.  The core update waits for the det pass, which
+  // reads the core populations, and runs beside the spawning, which does not
+  // read populations.  A failing record or wait invalidates the capture, which
+  // ending the capture reports.
+  if (branch) {
+    (void)(cudaEventRecord(E.ev_fork, s));
+    (void)(cudaStreamWaitEvent(aux, E.ev_fork, 0));
+    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, aux>>>(P, cur);
     if (with_core) {
-      k_core_locate<W><<<ncb, 256, 0, E.aux_stream>>>(P, cur);
-      k_core_spmv<<<(int)(((int64_t)P.ncore * 32 + 255) / 256), 256, 0, E.aux_stream>>>(P, cur);
+      k_core_locate<W><<<ncb, 256, 0, aux>>>(P, cur);
+      k_core_spmv<<<spmv_blocks, 256, 0, aux>>>(P, cur);
     }
-    if (branch) (void)(cudaEventRecord(E.ev_join, E.aux_stream));
-    k_det_pass<W, SYS><<<kScanBlocks, kScanThreads, 0, s>>>(P, cur);
-    k_scan_partials_i64<<<1, 1024, 0, s>>>(P.part, kScanBlocks, st_field_i64(st, offsetof(DevState, natt)), st);
-    k_scan_apply<int64_t><<<kScanBlocks, kScanThreads, 0, s>>>(
-        P.natt, P.att_begin, st_field_i64(st, offsetof(DevState, ndet) + 8 * cur), P.part, st);
-    if (branch) (void)(cudaStreamWaitEvent(s, E.ev_join, 0));
-    if (with_core) k_core_apply<<<ncb, 256, 0, s>>>(P, cur);
+  }
+  mark(0);
+  k_det_pass<W, SYS><<<kScanBlocks, kDetThreads, 0, s>>>(P, cur);
+  mark(1);
+  mark(2);
+  if (branch) {
+    if (with_core) {
+      (void)(cudaEventRecord(E.ev_fork, s));
+      (void)(cudaStreamWaitEvent(aux, E.ev_fork, 0));
+      k_core_apply<<<ncb, 256, 0, aux>>>(P, cur);
+    }
+    (void)(cudaEventRecord(E.ev_join, aux));
+    mark(3);
   } else {
-    mark(0);
-    k_det_pass<W, SYS><<<kScanBlocks, kScanThreads, 0, s>>>(P, cur);
-    mark(1);
-    k_scan_partials_i64<<<1, 1024, 0, s>>>(P.part, kScanBlocks, st_field_i64(st, offsetof(DevState, natt)), st);
-    k_scan_apply<int64_t><<<kScanBlocks, kScanThreads, 0, s>>>(
-        P.natt, P.att_begin, st_field_i64(st, offsetof(DevState, ndet) + 8 * cur), P.part, st);
-    mark(2);
     if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, s>>>(P, cur);
     mark(3);
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, s>>>(P, cur);
-      k_core_spmv<<<(int)(((int64_t)P.ncore * 32 + 255) / 256), 256, 0, s>>>(P, cur);
+      k_core_spmv<<<spmv_blocks, 256, 0, s>>>(P, cur);
       k_core_apply<<<ncb, 256, 0, s>>>(P, cur);
     }
   }
   mark(4);
   k_attempt<W, SYS><<<E.attempt_grid, kAttemptThreads, attempt_smem_bytes<W, SYS>(), s>>>(P, cur);
   mark(5);
+  if (branch) (void)(cudaStreamWaitEvent(s, E.ev_join, 0));
   if (P.hash_merge) {
     mark(6);
     mark(7);
@@ -231,19 +232,23 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
   if (branch) {
     (void)cudaEventRecord(fork, s);
     (void)cudaStreamWaitEvent(aux, fork, 0);
+    if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
+    if (G.max_ncore > 0) {
+      kb_core_locate<W><<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
+      kb_core_spmv<<<dim3((unsigned)(((int64_t)G.max_ncore * 32 + 255) / 256), R), 256, 0, aux>>>(PP, cur);
+    }
   }
-  if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
-  if (G.max_ncore > 0) {
-    kb_core_locate<W><<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
-    kb_core_spmv<<<dim3((unsigned)(((int64_t)G.max_ncore * 32 + 255) / 256), R), 256, 0, aux>>>(PP, cur);
+  kb_det_pass<W, SYS><<<blocks(0), kDetThreads, 0, s>>>(PP, off(0), R, cur);
+  if (branch) {
+    if (G.max_ncore > 0) {
+      (void)cudaEventRecord(fork, s);
+      (void)cudaStreamWaitEvent(aux, fork, 0);
+      kb_core_apply<<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
+    }
+    (void)cudaEventRecord(join, aux);
   }
-  if (branch) (void)cudaEventRecord(join, aux);
-  kb_det_pass<W, SYS><<<blocks(0), kScanThreads, 0, s>>>(PP, off(0), R, cur);
-  kb_scan_natt<<<dim3(1, R), 1024, 0, s>>>(PP, off(0), R);
-  kb_scan_att<<<blocks(0), kScanThreads, 0, s>>>(PP, off(0), R, cur);
-  if (branch) (void)cudaStreamWaitEvent(s, join, 0);
-  if (G.max_ncore > 0) kb_core_apply<<<dim3(ncb, R), 256, 0, s>>>(PP, cur);
   kb_attempt<W, SYS><<<blocks(1), kAttemptThreads, attempt_smem_bytes<W, SYS>(), s>>>(PP, off(1), R, cur);
+  if (branch) (void)cudaStreamWaitEvent(s, join, 0);
   if (hash) {
     kb_match<W><<<blocks(2), kMatchThreads, 0, s>>>(PP, off(2), R, cur);
     kb_decide<W><<<blocks(5), kListThreads, 0, s>>>(PP, off(5), R, cur);

@@ -235,6 +235,7 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
       }
       m[u] = __ballot_sync(0xffffffffu, keep);
     }
+    if (threadIdx.x == 0) P.det_state[c] = 0ull;   // look-back of the next det pass
     if (lane == 0) {
       P.g_keep[g] = (uint64_t)m[0] | ((uint64_t)m[1] << 32);
       scnt[wid] = (uint32_t)(__popc(m[0]) + __popc(m[1]));
@@ -325,10 +326,10 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
   }
 }
 template <int W>
-__global__ void __launch_bounds__(kListThreads) k_decide(Params P, int cur) { d_decide<W>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+__global__ void __launch_bounds__(kListThreads, W == 8 ? 2 : 3) k_decide(Params P, int cur) { d_decide<W>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
 // the same for a replica of a batch (parameter blocks PP[replica])
 template <int W>
-__global__ void __launch_bounds__(kListThreads) kb_decide(const Params* PP, const int* off, int R, int cur) {
+__global__ void __launch_bounds__(kListThreads, W == 8 ? 2 : 3) kb_decide(const Params* PP, const int* off, int R, int cur) {
   __shared__ Params sP;
   __shared__ VGrid vg;
   if (!batch_block(PP, off, R, sP, vg)) return;

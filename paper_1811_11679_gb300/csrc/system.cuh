@@ -227,22 +227,31 @@ __device__ double h_double(const SysDev& s, const Key<W>& d, int i, int j, int a
   return ((n1 + n2) & 1) ? -v : v;
 }
 
-// <target|H|source>
+// <target|H|source> of two determinants that differ in two or four spin orbitals
 template <int W, int SYS>
-__device__ double h_elem(const SysDev& s, const Key<W>& src, const Key<W>& tgt) {
-  int nd = key_popc_xor<W>(src, tgt);
-  if (nd == 0) return h_diag<W, SYS>(s, src);
-  if (nd != 2 && nd != 4) return 0.0;
+__device__ double h_connected(const SysDev& s, const Key<W>& src, const Key<W>& tgt) {
   Key<W> from, to;
 #pragma unroll
   for (int j = 0; j < W; ++j) {
-    uint64_t x = src.w[j] ^ tgt.w[j];
+    const uint64_t x = src.w[j] ^ tgt.w[j];
     from.w[j] = x & src.w[j];
     to.w[j] = x & tgt.w[j];
   }
-  if (nd == 2) return h_single<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(to, 0));
+  int nd = 0;
+#pragma unroll
+  for (int j = 0; j < W; ++j) nd += __popcll(from.w[j]);
+  if (nd == 1) return h_single<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(to, 0));
   return h_double<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(from, 1), select_bit<W>(to, 0),
                           select_bit<W>(to, 1));
+}
+
+// <target|H|source>
+template <int W, int SYS>
+__device__ double h_elem(const SysDev& s, const Key<W>& src, const Key<W>& tgt) {
+  const int nd = key_popc_xor<W>(src, tgt);
+  if (nd == 0) return h_diag<W, SYS>(s, src);
+  if (nd != 2 && nd != 4) return 0.0;
+  return h_connected<W, SYS>(s, src, tgt);
 }
 
 template <int W>
