@@ -931,6 +931,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       P.t_keep = dalloc<uint32_t>(E, tiles);
       P.t_base = dalloc<unsigned long long>(E, tiles);
       P.occ_draw = dalloc<uint32_t>(E, cap);
+      P.core_move = dalloc<uint32_t>(E, cap);
       for (int l = 1; l < kEndLevels && (cap >> (2 * l)) > 0; ++l)
         P.s_end[l] = dalloc<uint64_t>(E, (size_t)end_stride(cap, l) * E.W);
     } else {

@@ -520,6 +520,7 @@ __device__ __forceinline__ void d_write(const Params& P, int cur, const VGrid vg
         P.pop[nxt][o] = pp[u];
         P.hdiag[nxt][o] = hh[u];
         P.flags[nxt][o] = ff[u] & F_CORE;
+        if (ff[u] & F_CORE) P.core_move[g * kGroup + b] = (uint32_t)o;
       }
     }
   }
