@@ -129,7 +129,8 @@ void set_grids(hande_batch* b) {
   const double f = b->scale > 0.0 ? b->scale : 2.0;
   for (auto& G : b->groups) {
     const Engine& E = *G.eng[0];
-    const int base[hande::kPlanPhases] = {hande::kScanBlocks, E.attempt_grid, E.attempt_grid * 4,
+    const int base[hande::kPlanPhases] = {hande::kScanBlocks, E.attempt_grid,
+                                          E.attempt_grid * (E.P.hash_merge ? 2 : 4),
                                           std::max(E.merge_warp_grid, 1), E.merge_grid, E.attempt_grid * 2,
                                           E.attempt_grid};
     const int by_att[hande::kPlanPhases] = {0, 1, 1, 0, 0, 0, 0};

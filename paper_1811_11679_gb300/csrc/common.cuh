@@ -259,10 +259,15 @@ __device__ __forceinline__ double log_series(double x) {
   }
   double s = __ddiv_rn(__dsub_rn(m, 1.0), __dadd_rn(m, 1.0));
   double z = __dmul_rn(s, s);
-  double p = __ddiv_rn(1.0, 23.0);
+  // 1 / (2 k + 1), rounded at compile time (a run-time divide each took most of
+  // the 4.5 us of the one-thread shift update)
+  constexpr double inv_odd[12] = {1.0,        1.0 / 3.0,  1.0 / 5.0,  1.0 / 7.0,  1.0 / 9.0,  1.0 / 11.0,
+                                  1.0 / 13.0, 1.0 / 15.0, 1.0 / 17.0, 1.0 / 19.0, 1.0 / 21.0, 1.0 / 23.0};
+  double p = inv_odd[11];
+#pragma unroll
   for (int k = 10; k >= 0; --k) {
     p = __dmul_rn(p, z);
-    p = __dadd_rn(p, __ddiv_rn(1.0, (double)(2 * k + 1)));
+    p = __dadd_rn(p, inv_odd[k]);
   }
   double lnm = __dmul_rn(__dmul_rn(2.0, s), p);
   return __dadd_rn(__dmul_rn((double)e, 0.69314718055994530942), lnm);

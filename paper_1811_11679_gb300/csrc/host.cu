@@ -908,8 +908,9 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     P.natt = dalloc<int64_t>(E, cap);
     P.att_begin = dalloc<int64_t>(E, cap);
     P.part = dalloc<int64_t>(E, kScanBlocks + 1);
-    P.det_state = dalloc<unsigned long long>(E, cap / kDetTile + 2);
-    CK(cudaMemsetAsync(P.det_state, 0, (cap / kDetTile + 2) * sizeof(unsigned long long), E.stream));
+    const size_t det_states = (size_t)(list_tiles(cap) + kDetTile);
+    P.det_state = dalloc<unsigned long long>(E, det_states);
+    CK(cudaMemsetAsync(P.det_state, 0, det_states * sizeof(unsigned long long), E.stream));
     P.s_key = dalloc<uint64_t>(E, (size_t)scap * E.W);
     P.s_amt = dalloc<int64_t>(E, scap);
     P.s_meta = dalloc<uint64_t>(E, scap);

@@ -413,7 +413,8 @@ __device__ __forceinline__ unsigned long long lookback_warp(DevState* st, unsign
 
 // One pass over the list: estimators, initiator flags, death, attempt counts and
 // their exclusive scan (att_begin), in tiles of 1024 entries taken in ticket
-// order.  The scan is chained through the tiles (look-back) instead of a second
+// order (smaller ones for a short list, so that its FP64 work spreads over the
+// SMs).  The scan is chained through the tiles (look-back) instead of a second
 // and third kernel over the counts: those cost 21 us of a 930 us iteration on
 // 2.3e6 determinants, and two launches of the 17 of a small one.  Entries
 // connected to the reference (a percent of a large list) are queued and their
@@ -435,17 +436,22 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
   __shared__ int64_t queue_n[kDetTile];  // and their populations before death
   __shared__ int s_qn, s_abort;
   __shared__ unsigned s_tile;
-  if (__syncthreads_or((int)st->error)) return;
   const int64_t n = st->ndet[cur];
   const int64_t t = st->iter + 1;
   const double S = st->shift;
+  // short lists in smaller tiles, down to 64 entries, as long as that makes at
+  // most 16 tiles, each with a block of its own (Hubbard ring: 10.7 -> 6.6 us;
+  // with up to 512 tiles lists of 1e5 entries took longer, 12 -> 17 us)
+  int64_t size = kDetTile;
+  while (size > 64 && n <= size / 2 * (vg.n < 16 ? vg.n : 16)) size >>= 1;
+  const int64_t tiles = (n + size - 1) / size;
+  if (__syncthreads_or((int)st->error) || vg.b >= tiles) return;   // no tile for this block
   const Key<W> d0 = ref_key<W>(P);
   const uint64_t* key = P.key[cur];
   int64_t* pop = P.pop[cur];
   const double* hd = P.hdiag[cur];
   uint8_t* fl = P.flags[cur];
   const int lane = (int)warp_lane(), wid = (int)(threadIdx.x >> 5);
-  const int64_t tiles = (n + kDetTile - 1) / kDetTile;
   if (vg.b == 0 && threadIdx.x == 0 && P.hash_merge) {   // counters of the spawning and the annihilation
     st->nbuckets = n / 64 + 1;
     st->sb = 64;
@@ -461,9 +467,12 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
       s_abort = 0;
     }
     __syncthreads();
-    const int64_t tile = s_tile, base = tile * kDetTile;
+    const int64_t tile = s_tile, base = tile * size, last = base + size < n ? base + size : n;
     if (tile >= tiles) break;
-    if (P.hash_merge && threadIdx.x < 32) P.g_new[tile * 16 + threadIdx.x] = 0u;   // and the groups behind the list
+    if (P.hash_merge) {   // survivor counts of the tile's groups (and of those behind the list)
+      const int64_t ge = tile == tiles - 1 ? (n / 1024 + 1) * 16 : (base + size) / 64;
+      for (int64_t g = base / 64 + threadIdx.x; g < ge; g += blockDim.x) P.g_new[g] = 0u;
+    }
     unsigned long long na[kDetItems], pre[kDetItems];
     // all loads of the thread's entries before the first use
     Key<W> kk[kDetItems];
@@ -473,7 +482,7 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
 #pragma unroll
     for (int u = 0; u < kDetItems; ++u) {
       const int64_t i = base + u * kDetThreads + threadIdx.x;
-      if (i < n) {
+      if (i < last) {
         kk[u] = load_key<W>(key, P.cap, i);
         pp[u] = pop[i];
         ff[u] = fl[i];
@@ -484,7 +493,7 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
     for (int u = 0; u < kDetItems; ++u) {
       const int64_t i = base + u * kDetThreads + threadIdx.x;
       na[u] = 0;
-      if (i < n) {
+      if (i < last) {
         const Key<W>& k = kk[u];
         const int64_t p = pp[u];
         const uint8_t f = ff[u] & F_CORE;
@@ -568,8 +577,9 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
 #pragma unroll
     for (int u = 0; u < kDetItems; ++u) {
       const int64_t i = base + u * kDetThreads + threadIdx.x;
-      if (i < n) P.att_begin[i] = (int64_t)(wpre[u * kDetWarps + wid] + pre[u]);
+      if (i < last) P.att_begin[i] = (int64_t)(wpre[u * kDetWarps + wid] + pre[u]);
     }
+    if (tiles <= vg.n) break;   // one tile for each block
   }
   const int64_t b = block_sum<int64_t>(nw, sh64);
   if (threadIdx.x == 0 && b) atomicAdd((unsigned long long*)&st->nw_pre, (unsigned long long)b);
@@ -1227,20 +1237,22 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
   // The offsets att_begin[base .. base + 32] of the next chunk are loaded while
   // the current chunk is processed.
   const int64_t span = (((natt + total_warps - 1) / total_warps) + 31) & ~(int64_t)31;
-  const int64_t gbeg = ((int64_t)vg.b * kAttemptWarps + wid) * span;
+  // one chunk per warp: chunks over all SMs first; longer spans stay together
+  const int64_t gbeg = (span <= 32 ? (int64_t)wid * vg.n + vg.b : (int64_t)vg.b * kAttemptWarps + wid) * span;
   const int64_t gend = gbeg + span < natt ? gbeg + span : natt;
   int64_t base = 0, av = INT64_MAX, av32_l = INT64_MAX;
   if (gbeg < gend) {
-    if (lane == 0) {
-      int64_t lo = 0, hi = n - 1;
-      while (lo < hi) {
-        int64_t mid = (lo + hi + 1) >> 1;
-        if (P.att_begin[mid] <= gbeg) lo = mid;
-        else hi = mid - 1;
-      }
-      base = lo;
+    // the last parent whose attempts begin at or before gbeg: 32 probes a step,
+    // one per lane (three dependent reads for a list of 4e3 instead of twelve)
+    int64_t lo = 0, hi = n;   // att_begin[lo] <= gbeg < att_begin[hi]
+    while (hi - lo > 1) {
+      const int64_t step = (hi - lo + 31) / 32, at = lo + step * (lane + 1);
+      const unsigned le = __ballot_sync(0xffffffffu, at < hi && P.att_begin[at] <= gbeg);
+      const int c = __popc(le);   // probes are ordered: the first c hold
+      if (lo + step * (c + 1) < hi) hi = lo + step * (c + 1);
+      lo += step * c;
     }
-    base = __shfl_sync(0xffffffffu, base, 0);
+    base = lo;
     load_window(P.att_begin, n, base, lane, av, av32_l);
   }
   for (int64_t gw = gbeg; gw < gend; gw += 32) {
@@ -1345,8 +1357,7 @@ __device__ __forceinline__ void d_bucket(const Params& P, const VGrid vg) {
   if (st->error) return;
   const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap, nb = st->nbuckets;
   // the det pass's look-back states, for the next iteration
-  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c * kDetTile < P.cap && c * kDetTile < nb * st->sb;
-       c += (int64_t)vg.n * blockDim.x)
+  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c < P.cap / kDetTile + kDetTile; c += (int64_t)vg.n * blockDim.x)
     P.det_state[c] = 0ull;
   for (int64_t s = (int64_t)vg.b * blockDim.x + threadIdx.x; s < ns; s += (int64_t)vg.n * blockDim.x) {
     const Key<W> k = load_key<W>(P.s_key, P.scap, s);

@@ -19,12 +19,12 @@
 //           entries' keep bits in one word; each representative: initiator
 //           rule, rounding, slot cleared, and if it survives its rank of
 //           arrival among the survivors inserted in front of the same 64
-//           entries.  The last block scans the group counts and closes the
-//           iteration (shift, record).
+//           entries.  The last block scans the group counts.
 //   place   survivors copied group by group.
 //   write   diagonal elements of the survivors; entries and survivors to their final places in the new list: an
 //           entry's place follows from the keep bits and the survivors in front
 //           of it, a survivor's rank in its group from counting smaller keys.
+//           One thread closes the iteration meanwhile (shift, record).
 // What bounds them: match by L2 sectors and latency (one thread per spawn, all
 // resident), decide and write by HBM, the diagonal elements by the FP64 unit
 // (their sums are ordered), which runs beside the copy of the other blocks.
@@ -62,6 +62,12 @@ __device__ __forceinline__ uint32_t hash_mask(const Params& P, int64_t ns) {
   return (uint32_t)(m - 1);
 }
 
+// The 32-element chunk of warp wid of a block in one round of the grid: in block
+// order, or (spread) to all blocks before any block gets a second one.
+__device__ __forceinline__ int64_t chunk_of(const VGrid vg, int wid, bool spread) {
+  return spread ? (int64_t)wid * vg.n + vg.b : (int64_t)vg.b * (blockDim.x >> 5) + wid;
+}
+
 // ------------------------------------------------------------------ match
 // How many of the node's keys a[4 b .. 4 b + 3] (those below index `valid`) are
 // below k; hit: one of them is k.  Every node is an aligned 32-byte sector per word.
@@ -97,14 +103,20 @@ __device__ __forceinline__ void d_match(const Params& P, int cur, const VGrid vg
   __shared__ uint64_t ssp[W * S];
   __shared__ uint32_t swarp[kMatchThreads / 32];
   DevState* st = P.st;
-  if (__syncthreads_or((int)st->error)) return;
   const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap;
-  if ((int64_t)vg.b * blockDim.x >= ns) return;
   const uint32_t n = (uint32_t)st->ndet[cur];
+  // every block stages search keys, so spawns spread over all blocks only when
+  // each block gets at least eight warps of them (UEG 1e6 walkers: 31 -> 28 us;
+  // small replicas of a batch: 17 -> 20 us, hence the limit)
+  const bool spread = ns >= (int64_t)vg.n * 256;
+  if (__syncthreads_or((int)st->error) || chunk_of(vg, 0, spread) * 32 >= ns) return;
   const uint64_t* key = P.key[cur];
   unsigned long long* pop = (unsigned long long*)P.pop[cur];
-  int top = 1;   // block ends of level `top` go to shared memory
-  while ((n >> (2 * top)) > (uint32_t)S) ++top;
+  // block ends of level `top` go to shared memory: at most S of them, and no more
+  // than an eighth of the spawns (every block stages them)
+  const uint32_t most = ns / 8 < S ? (uint32_t)(ns / 8) : (uint32_t)S;
+  int top = 1;
+  while ((n >> (2 * top)) > most && top < kEndLevels - 1) ++top;
   const int nsp = (int)(n >> (2 * top));
   for (int i = threadIdx.x; i < nsp; i += blockDim.x) {
 #pragma unroll
@@ -114,8 +126,8 @@ __device__ __forceinline__ void d_match(const Params& P, int cur, const VGrid vg
   const uint32_t mask = hash_mask(P, ns);
   const int lane = (int)warp_lane(), wid = (int)(threadIdx.x >> 5);
   const int64_t step = (int64_t)vg.n * blockDim.x;
-  for (int64_t s0 = (int64_t)vg.b * blockDim.x; s0 < ns; s0 += step) {
-    const int64_t s = s0 + threadIdx.x;
+  for (int64_t s0 = chunk_of(vg, 0, spread) * 32; s0 < ns; s0 += step) {
+    const int64_t s = s0 + (spread ? (int64_t)wid * vg.n : wid) * 32 + lane;
     bool rep = false;
     if (s < ns) {
       const Key<W> k = load_key<W>(P.s_key, P.scap, s);
@@ -206,9 +218,10 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
   __shared__ unsigned long long s_carry;
   __shared__ int s_last;
   DevState* st = P.st;
-  if (__syncthreads_or((int)st->error)) return;
   const int64_t n = st->ndet[cur], t = st->iter + 1, nu = st->nuniq;
-  const int64_t nct = list_tiles(n);
+  const int64_t nct = list_tiles(n), want = (nu + 31) / 32;
+  const int64_t active = nct > want ? nct : want;   // blocks with work
+  if (__syncthreads_or((int)st->error) || vg.b >= active) return;
   const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
   int64_t* pop = P.pop[cur];
   const uint8_t* fl = P.flags[cur];
@@ -235,7 +248,6 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
       }
       m[u] = __ballot_sync(0xffffffffu, keep);
     }
-    if (threadIdx.x == 0) P.det_state[c] = 0ull;   // look-back of the next det pass
     if (lane == 0) {
       P.g_keep[g] = (uint64_t)m[0] | ((uint64_t)m[1] << 32);
       scnt[wid] = (uint32_t)(__popc(m[0]) + __popc(m[1]));
@@ -254,7 +266,9 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
     }
     __syncthreads();
   }
-  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < nu; i += (int64_t)vg.n * blockDim.x) {
+  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < nct + kDetTile; i += (int64_t)vg.n * blockDim.x)
+    P.det_state[i] = 0ull;   // look-back of the next det pass
+  for (int64_t i = chunk_of(vg, wid, true) * 32 + lane; i < nu; i += (int64_t)vg.n * blockDim.x) {
     const int64_t s = P.u_spawn[i];
     const uint64_t meta = P.s_meta[s];
     const uint32_t lo = (uint32_t)meta, pos = (uint32_t)(meta >> 32);
@@ -276,11 +290,11 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
     if (tot) atomicAdd((unsigned long long*)&st->nw_post, (unsigned long long)tot);
   }
   // the last block of the run: exclusive scan of the tiles' entry and survivor
-  // counts, new list length, shift and record
+  // counts, new list length
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_last = atomicAdd(&st->done_ticket, 1u) == (unsigned)vg.n - 1u;
+    s_last = atomicAdd(&st->done_ticket, 1u) == (unsigned)(active < vg.n ? active : vg.n) - 1u;
     s_carry = 0;
   }
   __syncthreads();
@@ -321,8 +335,6 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
     st->nnew = nnew;
     st->ndet[cur ^ 1] = nd;
     if (nd > P.max_det) set_error(st, ERR_STATE_CAPACITY);
-    // (error word and sum from L2: other blocks wrote them during this kernel)
-    if (atomicOr(&st->error, 0u) == 0u) finalize_iteration(P, nd, (int64_t)atomicAdd((unsigned long long*)&st->nw_post, 0ull));
   }
 }
 template <int W>
@@ -381,10 +393,11 @@ template <int W>
 __device__ __forceinline__ void d_place(const Params& P, int cur, const VGrid vg) {
   __shared__ int s_last;
   DevState* st = P.st;
-  if (__syncthreads_or((int)st->error)) return;
-  const int64_t nu = st->nuniq;
+  const int64_t nu = st->nuniq, active = (nu + 31) / 32;
+  if (__syncthreads_or((int)st->error) || vg.b >= active) return;
   bool large = false;
-  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < nu; i += (int64_t)vg.n * blockDim.x) {
+  const int lane = (int)warp_lane(), wid = (int)(threadIdx.x >> 5);
+  for (int64_t i = chunk_of(vg, wid, true) * 32 + lane; i < nu; i += (int64_t)vg.n * blockDim.x) {
     const uint32_t rank = P.u_rank[i];
     if (rank == ~0u) continue;
     const int64_t s = P.u_spawn[i];
@@ -401,7 +414,7 @@ __device__ __forceinline__ void d_place(const Params& P, int cur, const VGrid vg
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_last = atomicAdd(&st->done_ticket, 1u) == (unsigned)vg.n - 1u;
+    s_last = atomicAdd(&st->done_ticket, 1u) == (unsigned)(active < vg.n ? active : vg.n) - 1u;
     if (s_last) {
       st->done_ticket = 0;
       s_last = atomicExch(&st->big_ticket, 0u) ? 1 : 0;
@@ -427,17 +440,25 @@ __global__ void __launch_bounds__(256) kb_place(const Params* PP, const int* off
 template <int W, int SYS>
 __device__ __forceinline__ void d_write(const Params& P, int cur, const VGrid vg) {
   __shared__ uint32_t hist[kGroups][kGroup];
+  __shared__ uint8_t occ[SYS == SYS_HUBBARD ? 1 : kOccMax][kListThreads];
   DevState* st = P.st;
-  if (__syncthreads_or((int)st->error)) return;
   const int nxt = cur ^ 1;
   const int64_t n = st->ndet[cur], nnew = st->nnew;
+  if (__syncthreads_or((int)st->error)) return;
+  // the iteration's end: nothing below reads what it changes
+  if (vg.b == vg.n - 1 && threadIdx.x == kListThreads - 1) finalize_iteration(P, st->ndet[nxt], st->nw_post);
   const int64_t nct = list_tiles(n);
   const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
   const uint64_t* key = P.key[cur];
   uint64_t* okey = P.key[nxt];
   // new determinants, one thread each (first: their diagonal elements take longest)
   const uint32_t lim = large_group(P);
-  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < nnew; i += (int64_t)vg.n * blockDim.x) {
+  // A warp's FP64 addition takes 64 cycles alone on an SM and 304 among 16: up to
+  // one chunk per block, chunks go to all blocks (molecule 1e5 walkers: 24 -> 18
+  // us).  Beyond that the first blocks take them while the others copy (molecule
+  // 1e7 walkers: 31 us, spread 44).
+  const bool spread = nnew <= (int64_t)vg.n * 32;
+  for (int64_t i = chunk_of(vg, wid, spread) * 32 + lane; i < nnew; i += (int64_t)vg.n * blockDim.x) {
     const uint32_t pos = P.n_pos[i];
     const Key<W> k = load_key<W>(P.b_key, P.scap, i);
     const int64_t g = pos / kGroup, c = pos / kListTile;
@@ -464,7 +485,7 @@ __device__ __forceinline__ void d_write(const Params& P, int cur, const VGrid vg
                       __popcll(P.g_keep[g] & ((1ull << (pos & (kGroup - 1))) - 1ull)) + rank;
     store_key<W>(okey, P.cap, o, k);
     P.pop[nxt][o] = P.b_amt[i];
-    P.hdiag[nxt][o] = __dsub_rn(h_diag<W, SYS>(P.sys, k), st->e_ref);
+    P.hdiag[nxt][o] = __dsub_rn(h_diag_listed<W, SYS>(P.sys, k, &occ[0][threadIdx.x], kListThreads), st->e_ref);
     P.flags[nxt][o] = 0;
   }
   // listed entries, one group of 64 per warp
