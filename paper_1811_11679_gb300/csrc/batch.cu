@@ -184,8 +184,9 @@ hande_status regroup(hande_batch* b) {
     good = good &&
            ok(cudaFuncSetAttribute(E.ops.batch_attempt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)E.ops.attempt_smem)) &&
-           ok(cudaFuncSetAttribute(E.ops.batch_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)E.merge_smem_bytes));
+           (E.P.hash_merge || ok(cudaFuncSetAttribute(E.ops.batch_merge_kernel,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)E.merge_smem_bytes)));
     if (E.merge_warp)
       good = good && ok(cudaFuncSetAttribute(E.ops.batch_merge_warp_kernel,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -35,7 +35,8 @@ enum : unsigned {
 };
 
 // ------------------------------------------------------------------ keys
-// A determinant: W 64-bit words, bit p = spin orbital p (p = 2*spatial + spin).
+// A determinant: W 64-bit words, bit p = spin orbital p (p = 2*spatial + spin);
+// W = 1, 2, 8, or 3 for 512-bit keys whose spin orbitals fit in 192 bits.
 // Order: unsigned big integer, word W-1 most significant.
 template <int W>
 struct Key {
@@ -216,25 +217,36 @@ __device__ __forceinline__ uint64_t splitmix_fold(uint64_t z) {
   z ^= z >> 31;
   return z;
 }
+// counter words h0(D), h1(D) of a determinant's random stream: the key words for
+// 64- and 128-bit keys, a SplitMix64 fold of the eight words of a 512-bit key
+// (those kept as W = 3 words have five zero words behind them)
+struct Fold {
+  uint64_t h0, h1;
+};
+template <int W>
+__device__ __forceinline__ Fold key_fold(const Key<W>& d) {
+  if (W <= 2) return {d.w[0], (W == 2) ? d.w[W - 1] : 0ull};
+  uint64_t p = 0x243F6A8885A308D3ull, q = 0x13198A2E03707344ull;
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    p = splitmix_fold(p ^ d.w[j]);
+    q = splitmix_fold(q ^ d.w[j]);
+  }
+#pragma unroll
+  for (int j = W; j < 8; ++j) {
+    p = splitmix_fold(p);
+    q = splitmix_fold(q);
+  }
+  return {p, q};
+}
 // stream of determinant D at iteration t, attempt a: counter (t, a, h0(D), h1(D)),
-// key (seed, replica); h = the key words for W <= 2, a SplitMix64 fold above.
+// key (seed, replica)
+__device__ __forceinline__ Words4 draw(uint64_t seed, uint64_t replica, int64_t t, uint64_t a, const Fold& f) {
+  return philox4x64_10((uint64_t)t, a, f.h0, f.h1, seed, replica);
+}
 template <int W>
 __device__ __forceinline__ Words4 draw(uint64_t seed, uint64_t replica, int64_t t, uint64_t a, const Key<W>& d) {
-  uint64_t h0, h1;
-  if (W <= 2) {
-    h0 = d.w[0];
-    h1 = (W == 2) ? d.w[W - 1] : 0ull;
-  } else {
-    uint64_t p = 0x243F6A8885A308D3ull, q = 0x13198A2E03707344ull;
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      p = splitmix_fold(p ^ d.w[j]);
-      q = splitmix_fold(q ^ d.w[j]);
-    }
-    h0 = p;
-    h1 = q;
-  }
-  return philox4x64_10((uint64_t)t, a, h0, h1, seed, replica);
+  return draw(seed, replica, t, a, key_fold<W>(d));
 }
 __device__ __forceinline__ uint64_t draw_index(uint64_t w, uint64_t n) { return __umul64hi(w, n); }
 __device__ __forceinline__ double draw_unit(uint64_t w) { return __dmul_rn((double)(w >> 11), 0x1p-53); }

@@ -66,12 +66,15 @@ constexpr int kPhases = 10;   // timed phases of one iteration
 
 Ops ops_w1(int kind);
 Ops ops_w2(int kind);
+Ops ops_w3(int kind);
 Ops ops_w8(int kind);
 
 struct Engine {
   Params P{};            // device pointers and run constants (kernel argument)
   Ops ops{};
-  int W = 1, kind = 0, nalpha = 0, nbeta = 0;
+  int W = 1;    // words of a key on the device
+  int KW = 1;   // words of a key at the C ABI (key_words)
+  int kind = 0, nalpha = 0, nbeta = 0;
   int device = 0;                     // CUDA device the context was created on
   cudaStream_t stream = nullptr;      // caller's stream
   cudaStream_t cap_stream = nullptr;  // private stream used for graph capture

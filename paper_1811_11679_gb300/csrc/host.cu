@@ -753,7 +753,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     if (q.excit_gen != 0 && !(q.excit_gen == 1 && s.kind == HANDE_UEG))
       throw Fail{HANDE_ERR_INVALID, "excit_gen must be 0, or 1 (proposal table) for the UEG"};
 
-    E.W = s.key_words;
+    E.KW = s.key_words;
     E.kind = s.kind;
     E.nalpha = s.nalpha;
     E.nbeta = s.nbeta;
@@ -762,7 +762,11 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       E.alloc = *allocator;
       E.has_alloc = true;
     }
-    E.ops = E.W == 1 ? ops_w1(s.kind) : (E.W == 2 ? ops_w2(s.kind) : ops_w8(s.kind));
+    // default annihilation: the flat hash path (32-bit list positions and spawn
+    // indices), one warp per bucket for a list that does not fit those
+    E.P.hash_merge = q.annihilation == 0 && q.state_capacity < ((int64_t)1 << 31) - 4 ? 1 : 0;
+    E.W = E.KW == 8 && E.P.hash_merge && 2 * s.norb <= 192 ? 3 : E.KW;
+    E.ops = E.W == 1 ? ops_w1(s.kind) : (E.W == 2 ? ops_w2(s.kind) : (E.W == 3 ? ops_w3(s.kind) : ops_w8(s.kind)));
     CK(cudaStreamCreateWithFlags(&E.cap_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&E.aux_stream, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&E.ev_fork, cudaEventDisableTiming));
@@ -795,9 +799,6 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     // on-chip tile: distinct new keys (TC, a power of two for the bitonic sort) and
     // main-list entries (SM) per bucket
     if (q.annihilation < 0 || q.annihilation > 2) throw Fail{HANDE_ERR_INVALID, "annihilation must be 0, 1 or 2"};
-    // default: the flat hash path (32-bit list positions and spawn indices),
-    // one warp per bucket for a list that does not fit those
-    P.hash_merge = q.annihilation == 0 && P.cap < ((int64_t)1 << 31) ? 1 : 0;
     E.merge_warp = !P.hash_merge && q.annihilation != 1;
     // block tiles: sized so that four 256-thread CTAs share an SM for 64- and
     // 128-bit keys (two for 512-bit keys).  Warp path (three 8-warp CTAs per SM,
@@ -805,7 +806,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     // at most 192 entries (64 and 96 for 512-bit keys), buckets sized for 1.5 x
     // the staging in expected spawns (most land on listed entries) and for half
     // the staging in distinct new keys; the buckets it defers go to block tiles.
-    P.tile_cap = E.W == 8 ? 256 : 512;
+    P.tile_cap = E.KW == 8 ? 256 : 512;
     P.seg_max = E.merge_warp ? E.ops.merge_warp_main : (E.W == 1 ? 768 : (E.W == 2 ? 512 : 256));
     P.warp_cap = E.ops.merge_warp_new;
     if (q.tile_capacity > 0) {
@@ -900,11 +901,12 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     // ---- device buffers
     const int64_t cap = P.cap, scap = P.scap;
     for (int b = 0; b < 2; ++b) {
-      P.key[b] = dalloc<uint64_t>(E, (size_t)cap * E.W);
+      P.key[b] = dalloc<uint64_t>(E, (size_t)cap * E.KW);   // also stages keys of KW words
       P.pop[b] = dalloc<int64_t>(E, cap);
       P.hdiag[b] = dalloc<double>(E, cap);
       P.flags[b] = dalloc<uint8_t>(E, cap);
     }
+    if (E.W > 2) P.fold = dalloc<uint64_t>(E, 2 * (size_t)cap);
     P.natt = dalloc<int64_t>(E, cap);
     P.att_begin = dalloc<int64_t>(E, cap);
     P.part = dalloc<int64_t>(E, kScanBlocks + 1);
@@ -960,14 +962,16 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     CK(cudaGetDevice(&dev));
     E.device = dev;
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    E.merge_smem_bytes = E.ops.merge_smem(P.tile_cap, P.seg_max);
-    CK(cudaFuncSetAttribute(E.ops.merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)E.merge_smem_bytes));
-    int per_sm = 0;
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, E.ops.merge_kernel, kMergeThreads,
-                                                     E.merge_smem_bytes));
-    if (per_sm < 1) throw Fail{HANDE_ERR_CUDA, "annihilation kernel does not fit on an SM"};
-    E.merge_grid = per_sm * nsm;
+    if (!P.hash_merge) {
+      E.merge_smem_bytes = E.ops.merge_smem(P.tile_cap, P.seg_max);
+      CK(cudaFuncSetAttribute(E.ops.merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)E.merge_smem_bytes));
+      int per_sm = 0;
+      CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, E.ops.merge_kernel, kMergeThreads,
+                                                       E.merge_smem_bytes));
+      if (per_sm < 1) throw Fail{HANDE_ERR_CUDA, "annihilation kernel does not fit on an SM"};
+      E.merge_grid = per_sm * nsm;
+    }
     if (E.merge_warp) {
       CK(cudaFuncSetAttribute(E.ops.merge_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)E.ops.merge_warp_smem));
@@ -1147,7 +1151,7 @@ hande_status hande_get_walkers(hande_ctx* ctx, uint64_t* keys, int64_t* pops, do
     if (nd > cap) return HANDE_ERR_CAPACITY;
     if (nd == 0) return HANDE_OK;
     if (!keys || !pops) return HANDE_ERR_INVALID;
-    const int W = E.W;
+    const int W = E.KW;
     // keys transposed on the device into the other list buffer (free between
     // iterations), then one copy
     uint64_t* stage = E.P.key[cur ^ 1];
@@ -1174,7 +1178,7 @@ hande_status hande_set_walkers(hande_ctx* ctx, const uint64_t* keys, const int64
   Engine& E = ctx->E;
   if (E.failed) return HANDE_ERR_STATE;
   return run_guarded(&E, [&]() -> hande_status {
-    const int W = E.W;
+    const int W = E.KW;
     if (n > E.P.max_det) throw Fail{HANDE_ERR_CAPACITY, "more walkers than state_capacity"};
     // the keys go to the other list buffer (free between iterations), are
     // checked there and transposed into the list's layout
@@ -1259,7 +1263,7 @@ hande_status hande_get_state(hande_ctx* ctx, hande_state* out, uint64_t* core_ke
     uint64_t* stage = E.P.key[E.cur ^ 1];
     E.ops.keys_to_aos(E, E.core_key, stage, out->ncore, out->ncore, E.stream);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(core_keys, stage, (size_t)out->ncore * E.W * 8, cudaMemcpyDeviceToHost, E.stream));
+    CK(cudaMemcpyAsync(core_keys, stage, (size_t)out->ncore * E.KW * 8, cudaMemcpyDeviceToHost, E.stream));
     CK(cudaStreamSynchronize(E.stream));
     return HANDE_OK;
   });
@@ -1286,7 +1290,7 @@ hande_status hande_set_state(hande_ctx* ctx, const hande_state* in, const uint64
       // check the keys (ascending, electron numbers, the reference among them)
       // in the other list buffer, then transpose them into the core's layout
       uint64_t* stage = E.P.key[cur ^ 1];
-      CK(cudaMemcpyAsync(stage, core_keys, (size_t)ncore * E.W * 8, cudaMemcpyHostToDevice, E.stream));
+      CK(cudaMemcpyAsync(stage, core_keys, (size_t)ncore * E.KW * 8, cudaMemcpyHostToDevice, E.stream));
       CK(cudaMemsetAsync(E.check_word, 0, sizeof(unsigned), E.stream));
       E.ops.check_keys(E, stage, ncore, E.check_word, E.stream);
       CK(cudaGetLastError());
@@ -1519,7 +1523,7 @@ hande_status hande_reference(hande_ctx* ctx, double* e_ref, uint64_t* key) {
   if (!ctx) return HANDE_ERR_INVALID;
   if (e_ref) *e_ref = ctx->E.e_ref;
   if (key)
-    for (int j = 0; j < ctx->E.W; ++j) key[j] = ctx->E.P.d0[j];
+    for (int j = 0; j < ctx->E.KW; ++j) key[j] = ctx->E.P.d0[j];
   return HANDE_OK;
 }
 

@@ -138,6 +138,7 @@ struct Params {
   // draw (top half of Philox word z) and the last keys of its blocks of 4^l
   // entries (s_end[l], word stride end_stride)
   uint32_t* occ_draw;
+  uint64_t* fold;        // W > 2: counter words h0, h1 of each determinant (stride cap)
   uint64_t* s_end[kEndLevels];
   // deterministic space
   int ncore;
@@ -510,7 +511,12 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
         }
         const bool init = !P.initiator || mag > P.init_thr || is0 || core;
         Words4 w{};
-        if (p != 0 || (P.hash_merge && P.real_amp)) w = draw<W>(P.seed, P.replica, t, kDetDraw, k);
+        const Fold h = key_fold<W>(k);
+        if (W > 2) {   // the spawning reads them for each of the entry's attempts
+          P.fold[i] = h.h0;
+          P.fold[P.cap + i] = h.h1;
+        }
+        if (p != 0 || (P.hash_merge && P.real_amp)) w = draw(P.seed, P.replica, t, kDetDraw, h);
         if (P.hash_merge) {
           P.occ_draw[i] = (uint32_t)(w.z >> 32);
           for (int l = 1; ((i + 1) & ((int64_t(1) << (2 * l)) - 1)) == 0 && l < kEndLevels; ++l)
@@ -1299,7 +1305,8 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
       const uint64_t a = (uint64_t)(g - abeg);
       const Key<W> k = load_key<W>(key, P.cap, par);
       const uint8_t f = fl[par];
-      const Words4 w = draw<W>(P.seed, P.replica, t, a, k);
+      const Fold h = W > 2 ? Fold{P.fold[par], P.fold[P.cap + par]} : key_fold<W>(k);
+      const Words4 w = draw(P.seed, P.replica, t, a, h);
       const Excitation<W> ex = generate<W, SYS>(P.sys, gt, k, w);
       if (SYS == SYS_UEG && P.smp_cap > 0) record_sample(P, natt, g, ex);
       if (ex.single) {

@@ -118,13 +118,20 @@ __global__ void k_sel_gather(Params P, int cur, uint64_t* core_key, int64_t ncor
 }
 
 // ------------------------------------------------------------------ launchers
+// the bucket annihilation (qmc.annihilation = 1, 2) is built for the API's key
+// widths only, not for W = 3
+template <int W>
+constexpr bool kBuckets = W != 3;
+
+template <int W, int SYS>
+void enqueue_buckets(Engine& E, int cur, cudaStream_t s, cudaEvent_t* ev);
+
 // One iteration.  With `ev` non-null, ev[k] is recorded before phase k and
 // ev[kPhases] after the last one (phases: det pass, attempt scan, split, core,
 // attempts, bucket scan, scatter, merge, new diagonals, finalize).
 template <int W, int SYS>
 void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_t* ev) {
   Params& P = E.P;
-  [[maybe_unused]] DevState* st = P.st;
   auto mark = [&](int k) {
     if (ev) cudaEventRecord(ev[k], s);
   };
@@ -142,7 +149,8 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
   if (branch) {
     (void)(cudaEventRecord(E.ev_fork, s));
     (void)(cudaStreamWaitEvent(aux, E.ev_fork, 0));
-    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, aux>>>(P, cur);
+    if constexpr (kBuckets<W>)
+      if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, aux>>>(P, cur);
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, aux>>>(P, cur);
       k_core_spmv<<<spmv_blocks, 256, 0, aux>>>(P, cur);
@@ -161,7 +169,8 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
     (void)(cudaEventRecord(E.ev_join, aux));
     mark(3);
   } else {
-    if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, s>>>(P, cur);
+    if constexpr (kBuckets<W>)
+      if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, s>>>(P, cur);
     mark(3);
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, s>>>(P, cur);
@@ -185,6 +194,18 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
     mark(10);
     return;
   }
+  if constexpr (!kBuckets<W>) return;
+  else enqueue_buckets<W, SYS>(E, cur, s, ev);
+}
+
+// The rest of an iteration with the bucket annihilation.
+template <int W, int SYS>
+void enqueue_buckets(Engine& E, int cur, cudaStream_t s, cudaEvent_t* ev) {
+  Params& P = E.P;
+  DevState* st = P.st;
+  auto mark = [&](int k) {
+    if (ev) cudaEventRecord(ev[k], s);
+  };
   k_bucket<W><<<E.attempt_grid * 4, 256, 0, s>>>(P);
   int64_t* nbk = st_field_i64(st, offsetof(DevState, nbuckets));
   k_scan_one<uint32_t, uint32_t><<<1, 1024, 0, s>>>(P.bcount, P.boff, nbk,
@@ -241,7 +262,8 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
   if (branch) {
     (void)cudaEventRecord(fork, s);
     (void)cudaStreamWaitEvent(aux, fork, 0);
-    if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
+    if constexpr (kBuckets<W>)
+      if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
     if (G.max_ncore > 0) {
       kb_core_locate<W><<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
       kb_core_spmv<<<dim3((unsigned)(((int64_t)G.max_ncore * 32 + 255) / 256), R), 256, 0, aux>>>(PP, cur);
@@ -265,6 +287,7 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
     kb_write<W, SYS><<<blocks(5), kListThreads, 0, s>>>(PP, off(5), R, cur);
     return;
   }
+  if constexpr (kBuckets<W>) {
   kb_bucket<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
   kb_scan_buckets<<<dim3(1, R), 1024, 0, s>>>(PP);
   kb_scatter<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
@@ -283,6 +306,7 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
   }
   kb_new_hdiag<W, SYS><<<blocks(6), 256, 0, s>>>(PP, off(6), R, cur);
   kb_finalize<<<dim3(1, R), 32, 0, s>>>(PP, cur);
+}
 }
 
 template <int W, int SYS>
@@ -325,11 +349,11 @@ void enqueue_sel_gather(Engine& E, int cur, uint64_t* core_key, int64_t ncore, c
 }
 
 // ------------------------------------------------------------------ walker-list transfer
-// keys of a host-supplied list (array of structures, word j of key i at i W + j):
+// keys of a host-supplied list (array of structures, word j of key i at i kw + j):
 // bit 0 a bit beyond the spin orbitals, bit 1 wrong electron numbers, bit 2 not
 // strictly ascending, bit 3 the reference present
 template <int W>
-__global__ void k_check_keys(const uint64_t* aos, int64_t n, int nspin, int nalpha, int nbeta, Key<W> d0,
+__global__ void k_check_keys(const uint64_t* aos, int64_t n, int kw, int nspin, int nalpha, int nbeta, Key<W> d0,
                              unsigned* out) {
   unsigned bits = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -337,18 +361,20 @@ __global__ void k_check_keys(const uint64_t* aos, int64_t n, int nspin, int nalp
     int na = 0, nb = 0;
 #pragma unroll
     for (int j = 0; j < W; ++j) {
-      k.w[j] = aos[i * W + j];
+      k.w[j] = aos[i * kw + j];
       const int lo = 64 * j;
       if (nspin - lo < 64 && (nspin - lo <= 0 ? k.w[j] != 0 : (k.w[j] >> (nspin - lo)) != 0)) bits |= 1u;
       na += __popcll(k.w[j] & 0x5555555555555555ull);
       nb += __popcll(k.w[j] & 0xAAAAAAAAAAAAAAAAull);
     }
+    for (int j = W; j < kw; ++j)
+      if (aos[i * kw + j]) bits |= 1u;
     if (na != nalpha || nb != nbeta) bits |= 2u;
     if (key_eq<W>(k, d0)) bits |= 8u;
     if (i > 0) {
       Key<W> pk;
 #pragma unroll
-      for (int j = 0; j < W; ++j) pk.w[j] = aos[(i - 1) * W + j];
+      for (int j = 0; j < W; ++j) pk.w[j] = aos[(i - 1) * kw + j];
       if (!key_lt<W>(pk, k)) bits |= 4u;
     }
   }
@@ -356,17 +382,18 @@ __global__ void k_check_keys(const uint64_t* aos, int64_t n, int nspin, int nalp
 }
 // array of structures <-> the list's structure of arrays (key word j at j cap + i)
 template <int W>
-__global__ void k_keys_to_soa(const uint64_t* aos, uint64_t* soa, int64_t n, int64_t cap) {
+__global__ void k_keys_to_soa(const uint64_t* aos, uint64_t* soa, int64_t n, int64_t cap, int kw) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
-    for (int j = 0; j < W; ++j) soa[(size_t)j * cap + i] = aos[i * W + j];
+    for (int j = 0; j < W; ++j) soa[(size_t)j * cap + i] = aos[i * kw + j];
   }
 }
 template <int W>
-__global__ void k_keys_to_aos(const uint64_t* soa, uint64_t* aos, int64_t n, int64_t cap) {
+__global__ void k_keys_to_aos(const uint64_t* soa, uint64_t* aos, int64_t n, int64_t cap, int kw) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
-    for (int j = 0; j < W; ++j) aos[i * W + j] = soa[(size_t)j * cap + i];
+    for (int j = 0; j < W; ++j) aos[i * kw + j] = soa[(size_t)j * cap + i];
+    for (int j = W; j < kw; ++j) aos[i * kw + j] = 0ull;
   }
 }
 template <int W>
@@ -374,15 +401,15 @@ void enqueue_check_keys(Engine& E, const uint64_t* aos, int64_t n, unsigned* out
   Key<W> d0;
 #pragma unroll
   for (int j = 0; j < W; ++j) d0.w[j] = E.P.d0[j];
-  k_check_keys<W><<<4 * 152, 256, 0, s>>>(aos, n, E.P.sys.nspin, E.nalpha, E.nbeta, d0, out);
+  k_check_keys<W><<<4 * 152, 256, 0, s>>>(aos, n, E.KW, E.P.sys.nspin, E.nalpha, E.nbeta, d0, out);
 }
 template <int W>
 void enqueue_keys_to_soa(Engine& E, const uint64_t* aos, uint64_t* soa, int64_t n, int64_t stride, cudaStream_t s) {
-  k_keys_to_soa<W><<<4 * 152, 256, 0, s>>>(aos, soa, n, stride);
+  k_keys_to_soa<W><<<4 * 152, 256, 0, s>>>(aos, soa, n, stride, E.KW);
 }
 template <int W>
 void enqueue_keys_to_aos(Engine& E, const uint64_t* soa, uint64_t* aos, int64_t n, int64_t stride, cudaStream_t s) {
-  k_keys_to_aos<W><<<4 * 152, 256, 0, s>>>(soa, aos, n, stride);
+  k_keys_to_aos<W><<<4 * 152, 256, 0, s>>>(soa, aos, n, stride, E.KW);
 }
 // core flags from given core keys (restart): every list entry's core bit is
 // cleared, then each core key is found by binary search and flagged
@@ -415,12 +442,10 @@ size_t merge_smem_w(int tc, int sm) {
 
 template <int W, int SYS>
 Ops make_ops() {
-  Ops o;
+  Ops o{};
   o.iteration = &enqueue_iteration<W, SYS>;
   o.iteration_batch = &enqueue_iteration_batch<W, SYS>;
   o.batch_attempt_kernel = (const void*)&kb_attempt<W, SYS>;
-  o.batch_merge_kernel = (const void*)&kb_merge<W, SYS>;
-  o.batch_merge_warp_kernel = (const void*)&kb_merge_warp<W, SYS>;
   o.hdiag = &enqueue_hdiag<W, SYS>;
   o.eref = &enqueue_eref<W, SYS>;
   o.csr_count = &enqueue_csr_count<W, SYS>;
@@ -433,12 +458,16 @@ Ops make_ops() {
   o.core_hash = &enqueue_core_hash<W>;
   o.sel_hist = &enqueue_sel_hist<W>;
   o.sel_flags = &enqueue_sel_flags<W>;
-  o.merge_smem = &merge_smem_w<W>;
-  o.merge_kernel = (const void*)&k_merge<W, SYS>;
-  o.merge_warp_kernel = (const void*)&k_merge_warp<W, SYS>;
-  o.merge_warp_smem = merge_warp_smem_bytes<W>();
-  o.merge_warp_main = MwDims<W>::kMain;
-  o.merge_warp_new = MwDims<W>::kNew;
+  if constexpr (kBuckets<W>) {
+    o.batch_merge_kernel = (const void*)&kb_merge<W, SYS>;
+    o.batch_merge_warp_kernel = (const void*)&kb_merge_warp<W, SYS>;
+    o.merge_smem = &merge_smem_w<W>;
+    o.merge_kernel = (const void*)&k_merge<W, SYS>;
+    o.merge_warp_kernel = (const void*)&k_merge_warp<W, SYS>;
+    o.merge_warp_smem = merge_warp_smem_bytes<W>();
+    o.merge_warp_main = MwDims<W>::kMain;
+    o.merge_warp_new = MwDims<W>::kNew;
+  }
   o.attempt_kernel = (const void*)&k_attempt<W, SYS>;
   o.attempt_smem = attempt_smem_bytes<W, SYS>();
   return o;

@@ -179,8 +179,8 @@ extern "C" hande_status hande_estimate_noalloc(hande_ctx* ctx, const uint64_t* d
     }
     scratch = static_cast<Partial*>(g_scratch[dev]);
   }
-  if (E.W == 1) dispatch<1>(E, d_keys, d_pops, n, d_out, scratch);
-  else if (E.W == 2) dispatch<2>(E, d_keys, d_pops, n, d_out, scratch);
+  if (E.KW == 1) dispatch<1>(E, d_keys, d_pops, n, d_out, scratch);
+  else if (E.KW == 2) dispatch<2>(E, d_keys, d_pops, n, d_out, scratch);
   else dispatch<8>(E, d_keys, d_pops, n, d_out, scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

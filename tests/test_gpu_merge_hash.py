@@ -63,3 +63,28 @@ def test_group_larger_than_the_counting_limit(make, tau, init_pop):
     _same_records(g, c)
     assert largest > 16 * 64
     g.close()
+
+
+@pytest.mark.parametrize("norb", [65, 96, 97])   # 130, 192 (three device words) and 194 bits (eight)
+def test_wide_keys_at_the_three_word_limit(norb):
+    sysd = inputs.ueg_system(10, norb, 1.0)
+    assert sysd["key_words"] == 8
+    q = inputs.qmc_params(tau=0.001, target_population=1e6, initiator=1, real_amplitudes=1, spawn_cutoff=0.1,
+                          init_pop=2000, seed=5, state_capacity=50_001, spawn_capacity=100_000)
+    g, c = hande.Hande(sysd, q), oracle.Oracle(sysd, q)
+    for it in range(12):
+        g.iterate(1)
+        c.iterate(1)
+        _same_lists(g, c, it + 1)
+    _same_records(g, c)
+    k, p, h, _ = g.walkers()
+    g2 = hande.Hande(sysd, q)
+    g2.set_walkers(k, p)
+    k2, p2, h2, _ = g2.walkers()
+    assert np.array_equal(k, k2) and np.array_equal(p, p2) and np.array_equal(h, h2)
+    bad = k.copy()
+    bad[-1, 7] |= np.uint64(1) << np.uint64(63)    # beyond the spin orbitals
+    with pytest.raises(hande.HandeError):
+        g2.set_walkers(bad, p)
+    g.close()
+    g2.close()
