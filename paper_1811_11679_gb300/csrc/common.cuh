@@ -82,13 +82,19 @@ __device__ __forceinline__ int key_popc_xor(const Key<W>& a, const Key<W>& b) {
   for (int j = 0; j < W; ++j) n += __popcll(a.w[j] ^ b.w[j]);
   return n;
 }
+// (the word is chosen by compares: indexing it would put the key in local memory)
 template <int W>
 __device__ __forceinline__ bool key_bit(const Key<W>& k, int p) {
-  return (k.w[p >> 6] >> (p & 63)) & 1ull;
+  uint64_t x = k.w[0];
+#pragma unroll
+  for (int j = 1; j < W; ++j) x = (p >> 6) == j ? k.w[j] : x;
+  return (x >> (p & 63)) & 1ull;
 }
 template <int W>
 __device__ __forceinline__ void key_flip(Key<W>& k, int p) {
-  k.w[p >> 6] ^= 1ull << (p & 63);
+  const uint64_t bit = 1ull << (p & 63);
+#pragma unroll
+  for (int j = 0; j < W; ++j) k.w[j] ^= W == 1 || (p >> 6) == j ? bit : 0ull;
 }
 // number of set bits strictly between spin orbitals p and q (fermionic sign)
 template <int W>
@@ -248,7 +254,10 @@ template <int W>
 __device__ __forceinline__ Words4 draw(uint64_t seed, uint64_t replica, int64_t t, uint64_t a, const Key<W>& d) {
   return draw(seed, replica, t, a, key_fold<W>(d));
 }
-__device__ __forceinline__ uint64_t draw_index(uint64_t w, uint64_t n) { return __umul64hi(w, n); }
+// floor(w n / 2^64), n < 2^32 (two 32-bit wide products)
+__device__ __forceinline__ uint32_t draw_index(uint64_t w, uint32_t n) {
+  return (uint32_t)(((w >> 32) * n + (((w & 0xffffffffull) * n) >> 32)) >> 32);
+}
 __device__ __forceinline__ double draw_unit(uint64_t w) { return __dmul_rn((double)(w >> 11), 0x1p-53); }
 
 // ------------------------------------------------------------------ natural log

@@ -887,6 +887,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     sd.hb_pair = upload(E, T.hb_pair);
     sd.hb_cum = upload(E, T.hb_cum);
     sd.hb_ent = upload(E, T.hb_ent);
+    sd.hb_ab = upload(E, T.hb_ab);
     for (int j = 1; j < sd.nel; ++j)
       for (int i = 0; i < j; ++i) T.pair_ij.push_back((uint16_t)(i | (j << 8)));
     sd.pair_ij = upload(E, T.pair_ij);

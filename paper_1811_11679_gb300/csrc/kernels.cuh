@@ -978,13 +978,14 @@ static __global__ void kb_core_apply(const Params* PP, int cur) {
 
 // ------------------------------------------------------------------ attempts
 // ------------------------------------------------------------------ attempts
-// Attempts are processed 32 per warp.  Lanes diverge on what an attempt
-// produces (nothing, a spawn, a molecular single needing an O(N) matrix
-// element), so the rare outcomes go through per-warp shared-memory queues and
-// are finished 32 at a time by full warps: singles (select the orbitals,
-// evaluate H_ia, weight, rounding) and spawns (bucket search, append to the
-// staging arrays).  Two CTAs share an SM: the shared memory below stays
-// under half of an SM's 228 KB for every key width and system.
+// Attempts are processed 32 per warp.  Most draws come to nothing (target
+// orbitals occupied or outside the basis), so the rest of an attempt goes through
+// per-warp shared-memory queues and is finished 32 at a time by full warps:
+// surviving draws (sign, matrix element, core test, amount, rounding) and
+// molecular singles (orbitals, O(N) matrix element).  What these spawn is
+// appended to the staging arrays at once, one counter update per 32.  Two CTAs
+// share an SM: the shared memory below stays under half of an SM's 228 KB up to
+// 192-bit keys.
 constexpr int kAttemptThreads = 512;
 constexpr int kAttemptWarps = kAttemptThreads / 32;
 constexpr int kQueue = 64;   // per-warp queue capacity (holds 31 + 32 entries)
@@ -996,11 +997,12 @@ template <int W, int SYS>
 __host__ __device__ constexpr size_t attempt_stage_bytes() {
   return (SYS == SYS_MOLECULE && W == 1) ? (size_t)kStagePairs * (16 + 2) : 0;
 }
-// per-warp queue bytes per entry: spawns (key, amount, flag) and, for
-// molecules, singles (parent, words w and z, occupied rank)
+// per-warp queue bytes per entry: draws (parent key, word w, orbitals, two
+// numbers of the generator, flags) and, for molecules, singles (parent, words w
+// and z, occupied rank)
 template <int W, int SYS>
 __host__ __device__ constexpr size_t attempt_queue_entry() {
-  return (size_t)(8 * W + 8 + 1) + (SYS == SYS_MOLECULE ? (size_t)(8 + 8 + 8 + 1) : 0);
+  return (size_t)(8 * W + 8 + 8 + 4 + 4 + 1) + (SYS == SYS_MOLECULE ? (size_t)(8 + 8 + 8 + 1) : 0);
 }
 template <int W, int SYS>
 __host__ __device__ inline size_t attempt_smem_bytes() {
@@ -1012,9 +1014,12 @@ struct AttemptQueues {
   uint64_t* sq_word;   // their Philox word w (rounding)
   uint64_t* sq_wz;     // word z (empty orbital)
   uint8_t* sq_ri;      // rank of the occupied orbital, draw_index(w.y, N)
-  uint64_t* pq_key;    // finished spawns: key words [W][kQueue]
-  int64_t* pq_amt;
-  uint8_t* pq_flg;
+  uint64_t* dq_key;    // surviving draws: parent key words [W][kQueue]
+  uint64_t* dq_word;   // Philox word w (rounding)
+  ushort4* dq_orb;     // p, q, a, b
+  uint32_t* dq_e;      // molecule: heat-bath entry; proposal table: q_A + [same] q_B
+  uint32_t* dq_Q;      // proposal table: Q
+  uint8_t* dq_flg;     // parent flags
 };
 
 // time-step search: the warp's largest |H| / p_gen into the running maximum
@@ -1047,64 +1052,73 @@ __device__ __forceinline__ int64_t spawn_amount(const Params& P, uint64_t famt, 
   return neg ? -(int64_t)q : (int64_t)q;
 }
 
-// the top `take` queued spawns of this warp to the staging arrays (meta: the
-// initiator bit; the annihilation adds the spawn's place)
+// the lanes' spawns (amt != 0) to the staging arrays (meta: the initiator bit;
+// the annihilation adds the spawn's place); whole warp
 template <int W>
-__device__ void flush_spawns(const Params& P, const AttemptQueues& Q, int& pq_n, int take) {
+__device__ __forceinline__ void append_spawns(const Params& P, const Key<W>& child, int64_t amt, uint8_t pf) {
   DevState* st = P.st;
   const int lane = (int)warp_lane();
+  const unsigned m = __ballot_sync(0xffffffffu, amt != 0);
+  if (m == 0) return;
   int64_t base = 0;
-  if (lane == 0) base = (int64_t)atomicAdd((unsigned long long*)&st->nspawn, (unsigned long long)take);
+  if (lane == 0) base = (int64_t)atomicAdd((unsigned long long*)&st->nspawn, (unsigned long long)__popc(m));
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (lane < take) {
-    const int e = pq_n - take + lane;
-    const int64_t slot = base + lane;
+  if (amt != 0) {
+    const int64_t slot = base + __popc(m & ((1u << lane) - 1u));
     if (slot < P.scap) {
-#pragma unroll
-      for (int j = 0; j < W; ++j) P.s_key[j * P.scap + slot] = Q.pq_key[j * kQueue + e];
-      P.s_amt[slot] = Q.pq_amt[e];
-      P.s_meta[slot] = Q.pq_flg[e];
+      store_key<W>(P.s_key, P.scap, slot, child);
+      P.s_amt[slot] = amt;
+      P.s_meta[slot] = (pf & F_INIT) ? 1u : 0u;
     } else {
       set_error(st, ERR_SPAWN_CAPACITY);
     }
   }
-  pq_n -= take;
-  __syncwarp();
 }
 
-template <int W>
-__device__ __forceinline__ void push_spawn(const Params& P, const AttemptQueues& Q, int& pq_n, bool have,
-                                           const Key<W>& child, int64_t amt, uint8_t initf) {
-  const unsigned m = __ballot_sync(0xffffffffu, have);
-  if (have) {
-    const int e = pq_n + __popc(m & ((1u << warp_lane()) - 1u));
+// the top `take` queued draws of this warp: excitation, core test, amount
+template <int W, int SYS>
+__device__ __forceinline__ void flush_draws(const Params& P, const AttemptQueues& Q, int& dq_n, int take) {
+  const int lane = (int)warp_lane();
+  Key<W> child;
+  int64_t amt = 0;
+  uint8_t f = 0;
+  double rmax = 0.0;
+  if (lane < take) {
+    const int e = dq_n - take + lane;
+    Key<W> k;
 #pragma unroll
-    for (int j = 0; j < W; ++j) Q.pq_key[j * kQueue + e] = child.w[j];
-    Q.pq_amt[e] = amt;
-    Q.pq_flg[e] = initf;
+    for (int j = 0; j < W; ++j) k.w[j] = Q.dq_key[j * kQueue + e];
+    f = Q.dq_flg[e];
+    const ushort4 o = Q.dq_orb[e];
+    const Excitation<W> ex = resolve<W, SYS>(P.sys, k, o.x, o.y, o.z, o.w, Q.dq_e[e], Q.dq_e[e], Q.dq_Q[e]);
+    child = ex.child;
+    if (ex.ok && !((f & F_CORE) && P.ncore > 0 && in_core<W>(P, child))) {
+      rmax = ex.rval;
+      amt = spawn_amount(P, ex.famt, ex.hneg, Q.dq_word[e], f);
+    }
   }
-  pq_n += __popc(m);
+  dq_n -= take;
   __syncwarp();
-  if (pq_n >= 32) flush_spawns<W>(P, Q, pq_n, 32);
+  if (P.tau_search) ratio_max(P, rmax);
+  append_spawns<W>(P, child, amt, f);
 }
 
 // the top `take` queued molecular singles: orbitals, H_ia, core test, weight,
 // rounding
 template <int W, int SYS>
-__device__ void flush_singles(const Params& P, const AttemptQueues& Q, int& sq_n, int& pq_n, int take,
-                              const uint64_t* key, const uint8_t* fl) {
+__device__ void flush_singles(const Params& P, const AttemptQueues& Q, int& sq_n, int take, const uint64_t* key,
+                              const uint8_t* fl) {
   const int lane = (int)warp_lane();
-  bool have = false;
   Key<W> child;
   int64_t amt = 0;
-  uint8_t initf = 0;
+  uint8_t f = 0;
   double rmax = 0.0;
   if (lane < take) {
     const int e = sq_n - take + lane;
     const int64_t par = Q.sq_par[e];
     const uint64_t u = Q.sq_word[e];
     const Key<W> k = load_key<W>(key, P.cap, par);
-    const uint8_t f = fl[par];
+    f = fl[par];
     int i = 0, a = 0;
     const bool drawn = single_orbitals<W>(P.sys, k, Q.sq_ri[e], Q.sq_wz[e], i, a);
     child = k;
@@ -1115,14 +1129,12 @@ __device__ void flush_singles(const Params& P, const AttemptQueues& Q, int& sq_n
       if (P.tau_search) rmax = __dmul_rn(fabs(hij), P.sys.inv_single[i & 1]);
       const uint64_t famt = fixed_amount(abs_bits(hij), dbl_bits(P.sys.c_single[i & 1]), P.sys.half);
       amt = spawn_amount(P, famt, sign_bit(hij), u, f);
-      initf = (f & F_INIT) ? 1 : 0;
-      have = amt != 0;
     }
   }
   sq_n -= take;
   __syncwarp();
   if (P.tau_search) ratio_max(P, rmax);
-  push_spawn<W>(P, Q, pq_n, have, child, amt, initf);
+  append_spawns<W>(P, child, amt, f);
 }
 
 // largest i < n with a[i] <= x, given a[known] <= x (a non-decreasing):
@@ -1159,8 +1171,7 @@ __device__ __forceinline__ void load_window(const int64_t* a, int64_t n, int64_t
 // rejected one: the UEG matrix element depends only on the four momenta):
 // w = |H| / p(A | row) with |H| = |v(k_I - k_A) - [same spin] v(k_I - k_B)|,
 // v(q) = 4 pi / (Omega |q|^2), q = 0 terms omitted.
-template <int W>
-__device__ __forceinline__ void record_sample(const Params& P, int64_t natt, int64_t g, const Excitation<W>& ex) {
+__device__ __forceinline__ void record_sample(const Params& P, int64_t natt, int64_t g, const Draw& ex) {
   const int64_t stride = (natt + P.smp_cap - 1) / P.smp_cap;
   if (stride < 1 || g % stride != 0) return;
   const int64_t slot = g / stride;
@@ -1198,11 +1209,17 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
   {
     unsigned char* p = att_smem + attempt_stage_bytes<W, SYS>();
     const size_t per = kQueue;
-    Q.pq_key = reinterpret_cast<uint64_t*>(p) + wid * per * W;
+    Q.dq_key = reinterpret_cast<uint64_t*>(p) + wid * per * W;
     p += kAttemptWarps * per * 8 * W;
-    Q.pq_amt = reinterpret_cast<int64_t*>(p) + wid * per;
+    Q.dq_word = reinterpret_cast<uint64_t*>(p) + wid * per;
     p += kAttemptWarps * per * 8;
-    Q.pq_flg = reinterpret_cast<uint8_t*>(p) + wid * per;
+    Q.dq_orb = reinterpret_cast<ushort4*>(p) + wid * per;
+    p += kAttemptWarps * per * 8;
+    Q.dq_e = reinterpret_cast<uint32_t*>(p) + wid * per;
+    p += kAttemptWarps * per * 4;
+    Q.dq_Q = reinterpret_cast<uint32_t*>(p) + wid * per;
+    p += kAttemptWarps * per * 4;
+    Q.dq_flg = reinterpret_cast<uint8_t*>(p) + wid * per;
     p += kAttemptWarps * per;   // a multiple of 8 bytes
     Q.sq_par = nullptr;
     Q.sq_word = Q.sq_wz = nullptr;
@@ -1235,7 +1252,7 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
   __syncthreads();
   const int lane = (int)warp_lane();
   const int64_t total_warps = (int64_t)vg.n * kAttemptWarps;
-  int sq_n = 0, pq_n = 0;   // warp-uniform queue lengths
+  int sq_n = 0, dq_n = 0;   // warp-uniform queue lengths
   // each warp owns one contiguous span of attempts, taken in chunks of 32.
   // Parents are monotone in the attempt index: with base = the parent of a
   // chunk's first attempt, the chunk's parents lie in base .. base + 31 unless
@@ -1294,57 +1311,54 @@ __device__ __forceinline__ void d_attempt(const Params& P, int cur, const VGrid 
       par = gallop_last_le(P.att_begin, base + 31, n, g);
       abeg = P.att_begin[par];
     }
-    bool have = false, single = false;
-    Key<W> child;
-    int64_t amt = 0;
-    uint8_t initf = 0;
-    uint64_t word = 0, wz = 0;
-    uint8_t ri = 0;
-    double rmax = 0.0;
+    Draw ex;
+    ex.ok = ex.single = false;
+    Key<W> k;
+    Words4 w;
+    uint8_t f = 0;
     if (g < gend) {
-      const uint64_t a = (uint64_t)(g - abeg);
-      const Key<W> k = load_key<W>(key, P.cap, par);
-      const uint8_t f = fl[par];
+      k = load_key<W>(key, P.cap, par);
+      f = fl[par];
       const Fold h = W > 2 ? Fold{P.fold[par], P.fold[P.cap + par]} : key_fold<W>(k);
-      const Words4 w = draw(P.seed, P.replica, t, a, h);
-      const Excitation<W> ex = generate<W, SYS>(P.sys, gt, k, w);
+      w = draw(P.seed, P.replica, t, (uint64_t)(g - abeg), h);
+      ex = generate<W, SYS>(P.sys, gt, k, w);
       if (SYS == SYS_UEG && P.smp_cap > 0) record_sample(P, natt, g, ex);
-      if (ex.single) {
-        single = true;
-        word = w.w;
-        wz = w.z;
-        ri = (uint8_t)draw_index(w.y, (uint64_t)P.sys.nel);
-      } else if (ex.ok && !((f & F_CORE) && P.ncore > 0 && in_core<W>(P, ex.child))) {
-        rmax = fmax(rmax, ex.rval);
-        amt = spawn_amount(P, ex.famt, ex.hneg, w.w, f);
-        child = ex.child;
-        initf = (f & F_INIT) ? 1 : 0;
-        have = amt != 0;
-      }
     }
     if (SYS == SYS_MOLECULE) {
-      const unsigned sm = __ballot_sync(0xffffffffu, single);
-      if (single) {
+      const unsigned sm = __ballot_sync(0xffffffffu, ex.single);
+      if (ex.single) {
         const int e = sq_n + __popc(sm & ((1u << lane) - 1u));
         Q.sq_par[e] = par;
-        Q.sq_word[e] = word;
-        Q.sq_wz[e] = wz;
-        Q.sq_ri[e] = ri;
+        Q.sq_word[e] = w.w;
+        Q.sq_wz[e] = w.z;
+        Q.sq_ri[e] = (uint8_t)draw_index(w.y, (uint32_t)P.sys.nel);
       }
       sq_n += __popc(sm);
-      __syncwarp();
     }
-    if (P.tau_search) ratio_max(P, rmax);
-    push_spawn<W>(P, Q, pq_n, have, child, amt, initf);
-    if (SYS == SYS_MOLECULE && sq_n >= 32)
-      flush_singles<W, SYS>(P, Q, sq_n, pq_n, 32, key, fl);
+    const unsigned dm = __ballot_sync(0xffffffffu, ex.ok);
+    if (ex.ok) {
+      const int e = dq_n + __popc(dm & ((1u << lane) - 1u));
+#pragma unroll
+      for (int j = 0; j < W; ++j) Q.dq_key[j * kQueue + e] = k.w[j];
+      Q.dq_word[e] = w.w;
+      Q.dq_orb[e] = make_ushort4((unsigned short)ex.p, (unsigned short)ex.q, (unsigned short)ex.a, (unsigned short)ex.b);
+      if (SYS == SYS_MOLECULE) Q.dq_e[e] = ex.entry;
+      if (SYS == SYS_UEG) {
+        Q.dq_e[e] = ex.pqa + ex.pqb;
+        Q.dq_Q[e] = ex.pQ;
+      }
+      Q.dq_flg[e] = f;
+    }
+    dq_n += __popc(dm);
+    __syncwarp();
+    if (dq_n >= 32) flush_draws<W, SYS>(P, Q, dq_n, 32);
+    if (SYS == SYS_MOLECULE && sq_n >= 32) flush_singles<W, SYS>(P, Q, sq_n, 32, key, fl);
   }
-  if (SYS == SYS_MOLECULE && sq_n > 0)
-    flush_singles<W, SYS>(P, Q, sq_n, pq_n, sq_n, key, fl);
-  if (pq_n > 0) flush_spawns<W>(P, Q, pq_n, pq_n);
+  if (dq_n > 0) flush_draws<W, SYS>(P, Q, dq_n, dq_n);
+  if (SYS == SYS_MOLECULE && sq_n > 0) flush_singles<W, SYS>(P, Q, sq_n, sq_n, key, fl);
 }
 template <int W, int SYS>
-__global__ void __launch_bounds__(kAttemptThreads) k_attempt(Params P, int cur) { d_attempt<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+__global__ void __launch_bounds__(kAttemptThreads, W == 8 ? 1 : 2) k_attempt(Params P, int cur) { d_attempt<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
 // the same for replica blockIdx.y of a batch (parameter blocks PP[replica])
 // (two blocks per SM as for the single-run kernel: the shared-memory parameter
 // block would otherwise raise the register count past that)

@@ -50,6 +50,7 @@ struct SysDev {
   const int4* hb_pair;
   const uint64_t* hb_cum;
   const ulonglong2* hb_ent;
+  const uint16_t* hb_ab;   // a | b << 8 of each entry, for the occupancy test
   const uint16_t* hb_guide;
   uint32_t psingle_thr;
   double p_single, p_double;
@@ -375,13 +376,20 @@ __device__ double h_elem(const SysDev& s, const Key<W>& src, const Key<W>& tgt) 
   return h_connected<W, SYS>(s, src, tgt);
 }
 
+// One draw of a generator, before the work that only a possible spawn needs.
+struct Draw {
+  bool ok;               // a connected determinant was drawn (the target orbitals are empty)
+  bool single;           // a molecular single: its orbitals are left to the caller
+  int p, q, a, b;        // electrons p < q (Hubbard: p) to orbitals a, b (Hubbard: a; UEG: a of p's spin)
+  uint32_t entry;        // molecule: heat-bath entry
+  int prow, pA;          // proposal table: the row and particle orbital drawn (prow < 0: none)
+  uint32_t pqa, pqb, pQ; //   the drawn weights q_A, [same spin] q_B and the row total Q
+};
+// What a draw spawns.
 template <int W>
 struct Excitation {
-  bool ok;               // a connected child with H != 0 was drawn
-  bool single;           // a molecular single: chosen only, its orbitals and H_ia left to the caller
+  bool ok;               // H_child,parent != 0
   bool hneg;             // H_child,parent < 0
-  int prow, pA;          // proposal table: the row and particle orbital drawn (prow < 0: none)
-  uint32_t pqa, pQ;      //   the drawn weight q_A and the row total Q
   double rval;           // |H| / p_gen = (|H| inv_a) inv_b when the system's want_r is set
   uint64_t famt;         // fixed-point amount of |H| tau / p_gen (floored or rounded)
   Key<W> child;
@@ -395,7 +403,7 @@ struct GenTabs {
 };
 
 // pair index P = j(j-1)/2 + i  ->  (i, j), i < j (tabulated)
-__device__ __forceinline__ void unrank_pair(const uint16_t* pair_ij, uint64_t P, int& i, int& j) {
+__device__ __forceinline__ void unrank_pair(const uint16_t* pair_ij, uint32_t P, int& i, int& j) {
   uint16_t v = pair_ij[P];
   i = v & 0xff;
   j = v >> 8;
@@ -430,7 +438,7 @@ __device__ __forceinline__ bool single_orbitals(const SysDev& s, const Key<W>& d
 #pragma unroll
   for (int j = 0; j < W; ++j) ne += __popcll(empty.w[j]);
   if (ne == 0) return false;
-  a = select_bit<W>(empty, (int)draw_index(wz, (uint64_t)ne));
+  a = select_bit<W>(empty, (int)draw_index(wz, (uint32_t)ne));
   return true;
 }
 
@@ -444,93 +452,70 @@ __device__ __forceinline__ void finish(Excitation<W>& e, const SysDev& s, double
   e.ok = true;
 }
 
-// One excitation drawn from Philox words w (Sec. 2.4 spawning): the child, the
-// sign of its matrix element and the fixed-point amount of |H| tau / p_gen.
-// A molecular single is only selected (e.single, e.si, e.sa); its O(N) matrix
-// element is left to the caller.
+// One excitation drawn from Philox words w (Sec. 2.4 spawning).  Three of four
+// to eight of nine draws end here (an orbital outside the basis or occupied), so
+// the sign, the matrix element and the amount are left to resolve(), which the
+// caller runs on full warps of surviving draws.
 template <int W, int SYS>
-__device__ Excitation<W> generate(const SysDev& s, const GenTabs& gt, const Key<W>& d, const Words4& w) {
-  Excitation<W> e;
+__device__ __forceinline__ Draw generate(const SysDev& s, const GenTabs& gt, const Key<W>& d, const Words4& w) {
+  Draw e;
   e.ok = false;
   e.single = false;
-  e.hneg = false;
-  e.famt = 0;
+  e.p = e.q = e.a = e.b = 0;
+  e.entry = 0;
   e.prow = -1;
-  e.rval = 0.0;
-  const int n = s.nel;
+  e.pA = 0;
+  e.pqa = e.pqb = e.pQ = 0;
+  const uint32_t n = (uint32_t)s.nel;
   if (SYS == SYS_HUBBARD) {
-    int p = select_bit<W>(d, (int)draw_index(w.x, (uint64_t)n));
-    int site = p >> 1, spin = p & 1;
+    e.p = select_bit<W>(d, (int)draw_index(w.x, n));
     // hop k uniform among the z of the site (chain: 0 right, 1 left)
-    int ns = __ldg(&s.nbr[site * s.z + (int)draw_index(w.y, (uint64_t)s.z)]);
+    const int ns = __ldg(&s.nbr[(e.p >> 1) * s.z + (int)draw_index(w.y, (uint32_t)s.z)]);
     if (ns < 0) return e;
-    int q = 2 * ns + spin;
-    if (key_bit<W>(d, q)) return e;
-    e.child = d;
-    key_flip<W>(e.child, p);
-    key_flip<W>(e.child, q);
-    finish<W>(e, s, h_single<W, SYS>(s, d, p, q), s.c_hub, s.inv_hub, 1.0);
+    e.a = 2 * ns + (e.p & 1);
+    e.ok = !key_bit<W>(d, e.a);
     return e;
   } else if (SYS == SYS_UEG) {
-    uint64_t npairs = (uint64_t)n * (n - 1) / 2;
     int ii, jj;
-    unrank_pair(gt.pair_ij, draw_index(w.y, npairs), ii, jj);
-    int p = select_bit<W>(d, ii), q = select_bit<W>(d, jj);
+    unrank_pair(gt.pair_ij, draw_index(w.y, n * (n - 1) / 2), ii, jj);
+    e.p = select_bit<W>(d, ii);
+    e.q = select_bit<W>(d, jj);
+    const int I = e.p >> 1, J = e.q >> 1, same = ((e.p ^ e.q) & 1) ? 0 : 1;
+    const uint32_t* cum = nullptr;
+    int A;
     if (s.ptab_cum) {
       // proposal table: A by inverse CDF over the integer weights of row
       // (I, J, same spin); p_gen = (q_A + [same] q_B) / (Q C(N,2)), exact
-      const int M = s.norb, I = p >> 1, J = q >> 1, same = ((p ^ q) & 1) ? 0 : 1;
-      const int row = (I * M + J) * 2 + same;
-      const uint32_t* cum = s.ptab_cum + (size_t)row * M;
+      const int M = s.norb, row = (I * M + J) * 2 + same;
+      cum = s.ptab_cum + (size_t)row * M;
       const uint32_t Q = __ldg(&cum[M - 1]);
       if (Q == 0) return e;
-      const uint64_t x = draw_index(w.z, (uint64_t)Q);
+      const uint32_t x = (uint32_t)draw_index(w.z, Q);
       int lo = 0, hi = M - 1;   // the first A whose cumulative weight exceeds x
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if ((uint64_t)__ldg(&cum[mid]) > x) hi = mid;
+        if (__ldg(&cum[mid]) > x) hi = mid;
         else lo = mid + 1;
       }
-      const int A = lo;
-      int4 kp = __ldg(&s.kvec[I]), kq = __ldg(&s.kvec[J]), ka = __ldg(&s.kvec[A]);
-      int bx = kp.x + kq.x - ka.x, by = kp.y + kq.y - ka.y, bz = kp.z + kq.z - ka.z;
-      if (bx < -s.nmax || bx > s.nmax || by < -s.nmax || by > s.nmax || bz < -s.nmax || bz > s.nmax) return e;
-      const int B = __ldg(&s.klookup[((bx + s.nmax) * s.side + (by + s.nmax)) * s.side + (bz + s.nmax)]);
-      if (B < 0) return e;   // weight 0: not drawn
-      const uint32_t qa = __ldg(&cum[A]) - (A > 0 ? __ldg(&cum[A - 1]) : 0u);
-      const uint32_t qb = same ? __ldg(&cum[B]) - (B > 0 ? __ldg(&cum[B - 1]) : 0u) : 0u;
-      e.prow = row;
-      e.pA = A;
-      e.pqa = qa;
+      A = lo;
       e.pQ = Q;
-      const int a = 2 * A + (p & 1), b = 2 * B + (q & 1);
-      if (a == b || key_bit<W>(d, a) || key_bit<W>(d, b)) return e;
-      const int lo2 = a < b ? a : b, hi2 = a < b ? b : a;
-      e.child = d;
-      key_flip<W>(e.child, p);
-      key_flip<W>(e.child, q);
-      key_flip<W>(e.child, a);
-      key_flip<W>(e.child, b);
-      const double inv_b = __ddiv_rn((double)Q, (double)(qa + qb));
-      finish<W>(e, s, h_double<W, SYS>(s, d, p, q, lo2, hi2), __dmul_rn(s.c_tab, inv_b), s.inv_tab, inv_b);
-      return e;
+      e.pA = A;
+    } else {
+      A = (int)draw_index(w.z, (uint32_t)s.norb);
     }
-    int A = (int)draw_index(w.z, (uint64_t)s.norb);
-    int a = 2 * A + (p & 1);
-    int4 kp = __ldg(&s.kvec[p >> 1]), kq = __ldg(&s.kvec[q >> 1]), ka = __ldg(&s.kvec[A]);
-    int bx = kp.x + kq.x - ka.x, by = kp.y + kq.y - ka.y, bz = kp.z + kq.z - ka.z;
+    const int4 kp = __ldg(&s.kvec[I]), kq = __ldg(&s.kvec[J]), ka = __ldg(&s.kvec[A]);
+    const int bx = kp.x + kq.x - ka.x, by = kp.y + kq.y - ka.y, bz = kp.z + kq.z - ka.z;
     if (bx < -s.nmax || bx > s.nmax || by < -s.nmax || by > s.nmax || bz < -s.nmax || bz > s.nmax) return e;
-    int B = __ldg(&s.klookup[((bx + s.nmax) * s.side + (by + s.nmax)) * s.side + (bz + s.nmax)]);
-    if (B < 0) return e;
-    int b = 2 * B + (q & 1);
-    if (a == b || key_bit<W>(d, a) || key_bit<W>(d, b)) return e;
-    int lo = a < b ? a : b, hi = a < b ? b : a;
-    e.child = d;
-    key_flip<W>(e.child, p);
-    key_flip<W>(e.child, q);
-    key_flip<W>(e.child, a);
-    key_flip<W>(e.child, b);
-    finish<W>(e, s, h_double<W, SYS>(s, d, p, q, lo, hi), s.c_ueg[(p ^ q) & 1], s.inv_ueg[(p ^ q) & 1], 1.0);
+    const int B = __ldg(&s.klookup[((bx + s.nmax) * s.side + (by + s.nmax)) * s.side + (bz + s.nmax)]);
+    if (B < 0) return e;   // (proposal table: weight 0, not drawn)
+    if (cum) {
+      e.pqa = __ldg(&cum[A]) - (A > 0 ? __ldg(&cum[A - 1]) : 0u);
+      e.pqb = same ? __ldg(&cum[B]) - (B > 0 ? __ldg(&cum[B - 1]) : 0u) : 0u;
+      e.prow = (I * s.norb + J) * 2 + same;
+    }
+    e.a = 2 * A + (e.p & 1);
+    e.b = 2 * B + (e.q & 1);
+    e.ok = e.a != e.b && !key_bit<W>(d, e.a) && !key_bit<W>(d, e.b);
     return e;
   } else {
     if ((uint32_t)(w.x >> 32) < s.psingle_thr) {
@@ -539,11 +524,11 @@ __device__ Excitation<W> generate(const SysDev& s, const GenTabs& gt, const Key<
       e.single = true;
       return e;
     }
-    uint64_t npairs = (uint64_t)n * (n - 1) / 2;
     int ii, jj;
-    unrank_pair(gt.pair_ij, draw_index(w.y, npairs), ii, jj);
-    int p = select_bit<W>(d, ii), q = select_bit<W>(d, jj);
-    const int4 pr = gt.hb_pair[q * (q - 1) / 2 + p];   // {start, len, guide offset, guide bits}
+    unrank_pair(gt.pair_ij, draw_index(w.y, n * (n - 1) / 2), ii, jj);
+    e.p = select_bit<W>(d, ii);
+    e.q = select_bit<W>(d, jj);
+    const int4 pr = gt.hb_pair[e.q * (e.q - 1) / 2 + e.p];   // {start, len, guide offset, guide bits}
     if (pr.y == 0) return e;
     // smallest k with w.z < cum[k] among the first len - 1 entries, else the last
     const uint64_t t = w.z >> (64 - pr.w);
@@ -553,25 +538,65 @@ __device__ Excitation<W> generate(const SysDev& s, const GenTabs& gt, const Key<
       if (__ldg(&s.hb_cum[pr.x + mid]) <= w.z) lo = mid + 1;
       else hi = mid;
     }
-    const ulonglong2 ent = __ldg(&s.hb_ent[pr.x + lo]);
-    const int meta = (int)ent.y;
-    const int a = meta & 0xff, b = (meta >> 8) & 0xff;
-    if (key_bit<W>(d, a) || key_bit<W>(d, b)) return e;
-    // Slater-Condon sign of p -> a, then q -> b on the updated string
-    Key<W> tmp = d;
-    const int n1 = key_between<W>(tmp, p, a);
-    key_flip<W>(tmp, p);
-    key_flip<W>(tmp, a);
-    const int n2 = key_between<W>(tmp, q, b);
-    key_flip<W>(tmp, q);
-    key_flip<W>(tmp, b);
-    e.child = tmp;
-    e.famt = ent.x;
-    e.hneg = (((meta >> 16) ^ n1 ^ n2) & 1) != 0;
-    e.ok = true;
-    if (s.want_r) e.rval = __ldg(&s.hb_R[pr.x + lo]);
+    e.entry = (uint32_t)(pr.x + lo);
+    const int meta = __ldg(&s.hb_ab[e.entry]);
+    e.a = meta & 0xff;
+    e.b = meta >> 8;
+    e.ok = !key_bit<W>(d, e.a) && !key_bit<W>(d, e.b);
     return e;
   }
+}
+
+// The excitation of a surviving draw: child, sign, fixed-point amount.
+template <int W, int SYS>
+__device__ __forceinline__ Excitation<W> resolve(const SysDev& s, const Key<W>& d, int p, int q, int a, int b,
+                                                 uint32_t entry, uint32_t pq, uint32_t pQ) {
+  Excitation<W> e;
+  e.ok = false;
+  e.hneg = false;
+  e.famt = 0;
+  e.rval = 0.0;
+  e.child = d;
+  key_flip<W>(e.child, p);
+  key_flip<W>(e.child, a);
+  if (SYS == SYS_HUBBARD) {   // -t times the sign of p -> a (a is a neighbour by construction)
+    finish<W>(e, s, (key_between<W>(d, p, a) & 1) ? s.t : -s.t, s.c_hub, s.inv_hub, 1.0);
+  } else if (SYS == SYS_UEG) {
+    // Slater-Condon double p -> lo, q -> hi (momentum is conserved by
+    // construction); 4 pi / (Omega |k|^2) from the table of exchange kernels: the
+    // FP64 divides of evaluating it took half of the spawning kernel's time
+    const int lo = a < b ? a : b, hi = a < b ? b : a;
+    Key<W> tmp = d;
+    const int n1 = key_between<W>(tmp, p, lo);
+    key_flip<W>(tmp, p);
+    key_flip<W>(tmp, lo);
+    const int n2 = key_between<W>(tmp, q, hi);
+    key_flip<W>(e.child, q);
+    key_flip<W>(e.child, b);
+    const double* row = s.pair_diag + (size_t)(p >> 1) * s.norb;
+    double direct = 0.0, exch = 0.0;
+    if (!((p ^ lo) & 1) && !((q ^ hi) & 1)) direct = __ldg(&row[lo >> 1]);
+    if (!((p ^ hi) & 1) && !((q ^ lo) & 1)) exch = __ldg(&row[hi >> 1]);
+    const double v = __dsub_rn(direct, exch), h = ((n1 + n2) & 1) ? -v : v;
+    if (s.ptab_cum) {
+      const double inv_b = __ddiv_rn((double)pQ, (double)pq);
+      finish<W>(e, s, h, __dmul_rn(s.c_tab, inv_b), s.inv_tab, inv_b);
+    } else {
+      finish<W>(e, s, h, s.c_ueg[(p ^ q) & 1], s.inv_ueg[(p ^ q) & 1], 1.0);
+    }
+  } else {
+    // Slater-Condon sign of p -> a, then q -> b on the updated string
+    const ulonglong2 ent = __ldg(&s.hb_ent[entry]);
+    const int n1 = key_between<W>(d, p, a);
+    const int n2 = key_between<W>(e.child, q, b);
+    key_flip<W>(e.child, q);
+    key_flip<W>(e.child, b);
+    e.famt = ent.x;
+    e.hneg = ((((int)ent.y >> 16) ^ n1 ^ n2) & 1) != 0;
+    e.ok = true;
+    if (s.want_r) e.rval = __ldg(&s.hb_R[entry]);
+  }
+  return e;
 }
 
 }  // namespace hande
