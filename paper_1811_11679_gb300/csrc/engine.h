@@ -62,6 +62,7 @@ struct Ops {
   size_t attempt_smem;
 };
 
+constexpr int kPinRecords = 64;   // records read back through the page-locked block
 constexpr int kPhases = 10;   // timed phases of one iteration
 
 Ops ops_w1(int kind);
@@ -105,6 +106,7 @@ struct Engine {
   unsigned* check_word = nullptr;   // result word of the walker-list checks
   int64_t core_table_cap = 0;
   double e_ref = 0.0;
+  void* pin = nullptr;              // page-locked host block: DevState, then kPinRecords records
   // UEG proposal table (excit_gen = 1): cumulative weights on the device and
   // the drawable mask (host and device); the learned proposal, if attached
   uint32_t* ptab = nullptr;

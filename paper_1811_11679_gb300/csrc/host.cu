@@ -44,6 +44,8 @@ void release_all(Engine& E) {
     cudaStreamDestroy(E.aux_stream);
     E.aux_stream = nullptr;
   }
+  if (E.pin) cudaFreeHost(E.pin);
+  E.pin = nullptr;
   if (E.ev_fork) cudaEventDestroy(E.ev_fork);
   if (E.ev_join) cudaEventDestroy(E.ev_join);
   E.ev_fork = E.ev_join = nullptr;
@@ -423,12 +425,20 @@ void set_tau(Engine& E, double tau, bool to_device) {
                        cudaMemcpyHostToDevice, E.stream));
 }
 
-unsigned read_error(Engine& E) {
-  unsigned e = 0;
-  CK(cudaMemcpyAsync(&e, (char*)E.P.st + offsetof(DevState, error), sizeof(e), cudaMemcpyDeviceToHost, E.stream));
+// The device state in the page-locked block, after the stream's work (and after
+// any copies the caller enqueued before this): one synchronisation.  Reading
+// its words one by one into pageable memory cost a synchronisation each, about
+// 10 us of the host's time.
+const DevState& read_state(Engine& E) {
+  CK(cudaMemcpyAsync(E.pin, E.P.st, sizeof(DevState), cudaMemcpyDeviceToHost, E.stream));
   CK(cudaStreamSynchronize(E.stream));
-  return e;
+  return *static_cast<const DevState*>(E.pin);
 }
+Record* pin_records(Engine& E) {
+  return reinterpret_cast<Record*>(static_cast<char*>(E.pin) + ((sizeof(DevState) + 63) & ~size_t(63)));
+}
+
+unsigned read_error(Engine& E) { return read_state(E).error; }
 
 hande_status map_error(Engine& E, unsigned e) {
   if (!e) return HANDE_OK;
@@ -899,6 +909,8 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     sd.ptab_cum = nullptr;
     if (q.excit_gen == 1) proposal_init(E, T.kvec.data(), T.klookup.data(), sd.nmax, sd.side);
 
+    CK(cudaHostAlloc(&E.pin, ((sizeof(DevState) + 63) & ~size_t(63)) + kPinRecords * sizeof(Record), cudaHostAllocDefault));
+
     // ---- device buffers
     const int64_t cap = P.cap, scap = P.scap;
     for (int b = 0; b < 2; ++b) {
@@ -911,7 +923,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     P.natt = dalloc<int64_t>(E, cap);
     P.att_begin = dalloc<int64_t>(E, cap);
     P.part = dalloc<int64_t>(E, kScanBlocks + 1);
-    const size_t det_states = (size_t)(list_tiles(cap) + kDetTile);
+    const size_t det_states = (size_t)(list_tiles(cap) + 16);   // a short list has up to 16 smaller tiles
     P.det_state = dalloc<unsigned long long>(E, det_states);
     CK(cudaMemsetAsync(P.det_state, 0, det_states * sizeof(unsigned long long), E.stream));
     P.s_key = dalloc<uint64_t>(E, (size_t)scap * E.W);
@@ -1092,28 +1104,30 @@ hande_status hande_estimators(hande_ctx* ctx, hande_estimate* out, int max, int*
   if (n_out) *n_out = 0;
   if (E.failed) return HANDE_ERR_STATE;
   return run_guarded(&E, [&]() -> hande_status {
-    hande_status es = map_error(E, read_error(E));
-    if (es != HANDE_OK) return es;
     bool lost = false;
     if (E.host_iter - E.fetched > E.P.rec_cap) {
       E.fetched = E.host_iter - E.P.rec_cap;
       lost = true;
     }
-    int64_t avail = E.host_iter - E.fetched;
-    int64_t m = std::min<int64_t>(avail, max);
-    std::vector<Record> tmp((size_t)m);
+    const int64_t avail = E.host_iter - E.fetched;
+    const int64_t m = std::min<int64_t>(avail, max);
+    std::vector<Record> big;
+    Record* tmp = pin_records(E);
+    if (m > kPinRecords) {
+      big.resize((size_t)m);
+      tmp = big.data();
+    }
     if (m > 0) {   // the ring's slots from the first unread one: at most two contiguous runs
       const int64_t first = E.fetched % E.P.rec_cap;
       const int64_t run = std::min<int64_t>(m, E.P.rec_cap - first);
-      CK(cudaMemcpyAsync(tmp.data(), E.P.rec + first, (size_t)run * sizeof(Record), cudaMemcpyDeviceToHost,
-                         E.stream));
+      CK(cudaMemcpyAsync(tmp, E.P.rec + first, (size_t)run * sizeof(Record), cudaMemcpyDeviceToHost, E.stream));
       if (m > run)
-        CK(cudaMemcpyAsync(tmp.data() + run, E.P.rec, (size_t)(m - run) * sizeof(Record), cudaMemcpyDeviceToHost,
-                           E.stream));
+        CK(cudaMemcpyAsync(tmp + run, E.P.rec, (size_t)(m - run) * sizeof(Record), cudaMemcpyDeviceToHost, E.stream));
     }
-    CK(cudaStreamSynchronize(E.stream));
+    hande_status es = map_error(E, read_error(E));   // synchronises; the records came before it
+    if (es != HANDE_OK) return es;
     for (int64_t i = 0; i < m; ++i) {
-      const Record& r = tmp[(size_t)i];
+      const Record& r = tmp[i];
       hande_estimate& o = out[i];
       o.iter = r.iter;
       o.shift = r.shift;
@@ -1144,10 +1158,11 @@ hande_status hande_get_walkers(hande_ctx* ctx, uint64_t* keys, int64_t* pops, do
   Engine& E = ctx->E;
   if (E.failed) return HANDE_ERR_STATE;
   return run_guarded(&E, [&]() -> hande_status {
-    hande_status es = map_error(E, read_error(E));
-    if (es != HANDE_OK) return es;
     const int cur = E.cur;
-    int64_t nd = read_i64(E, offsetof(DevState, ndet) + 8 * cur);
+    const DevState& hs = read_state(E);
+    const int64_t nd = hs.ndet[cur];
+    hande_status es = map_error(E, hs.error);
+    if (es != HANDE_OK) return es;
     *n = nd;
     if (nd > cap) return HANDE_ERR_CAPACITY;
     if (nd == 0) return HANDE_OK;

@@ -1378,7 +1378,7 @@ __device__ __forceinline__ void d_bucket(const Params& P, const VGrid vg) {
   if (st->error) return;
   const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap, nb = st->nbuckets;
   // the det pass's look-back states, for the next iteration
-  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c < P.cap / kDetTile + kDetTile; c += (int64_t)vg.n * blockDim.x)
+  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c < P.cap / kDetTile + 16; c += (int64_t)vg.n * blockDim.x)
     P.det_state[c] = 0ull;
   for (int64_t s = (int64_t)vg.b * blockDim.x + threadIdx.x; s < ns; s += (int64_t)vg.n * blockDim.x) {
     const Key<W> k = load_key<W>(P.s_key, P.scap, s);

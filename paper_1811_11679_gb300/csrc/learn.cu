@@ -57,11 +57,12 @@ struct Learner {
   float *Z3 = nullptr, *dH = nullptr;
   float* wsum = nullptr;
   double* loss = nullptr;
-  unsigned* err = nullptr;
+  unsigned* err = nullptr;   // the word behind the loss
   // rows/targets/weights of a batch given through the C ABI (tests)
   int32_t *in_rows = nullptr, *in_tgt = nullptr;
   float* in_w = nullptr;
   float* probs = nullptr;
+  char* pin = nullptr;   // page-locked: a batch's rows, targets and weights, then the loss and the error word
   cudaGraphExec_t graph = nullptr;
 };
 
@@ -504,11 +505,12 @@ void learner_attach(Engine& E, const hande_learning& in) {
   L.Z3 = dalloc<float>(E, (size_t)L.rows_cap * M);
   L.dH = dalloc<float>(E, (size_t)L.S * H);
   L.wsum = dalloc<float>(E, 1);
-  L.loss = dalloc<double>(E, 1);
-  L.err = dalloc<unsigned>(E, 1);
-  L.in_rows = dalloc<int32_t>(E, L.S);
-  L.in_tgt = dalloc<int32_t>(E, L.S);
-  L.in_w = dalloc<float>(E, L.S);
+  L.loss = dalloc<double>(E, 2);
+  L.err = reinterpret_cast<unsigned*>(L.loss + 1);
+  L.in_rows = dalloc<int32_t>(E, 3 * (size_t)L.S);   // one upload for the three
+  L.in_tgt = L.in_rows + L.S;
+  L.in_w = reinterpret_cast<float*>(L.in_tgt + L.S);
+  CK(cudaHostAlloc((void**)&L.pin, 12 * (size_t)L.S + 16, cudaHostAllocDefault));
   L.probs = dalloc<float>(E, (size_t)L.S * M);
   // sample buffers of the spawning kernel
   E.P.smp_row = dalloc<int32_t>(E, L.S);
@@ -547,6 +549,10 @@ void learner_attach(Engine& E, const hande_learning& in) {
 void learner_release(Engine& E) {
   if (!E.learn) return;
   if (E.learn->graph) cudaGraphExecDestroy(E.learn->graph);
+  if (E.learn->pin) {
+    cudaStreamSynchronize(E.stream);
+    cudaFreeHost(E.learn->pin);
+  }
   delete E.learn;
   E.learn = nullptr;
 }
@@ -568,10 +574,13 @@ void learner_params(Engine& E, float* get, const float* set) {
 }
 
 // upload a batch of n <= S samples (rows, targets, weights; the rest weight 0)
+// through the page-locked block, one copy (the calls that use it synchronise
+// before they return, so the block is free again)
 static void upload_batch(Engine& E, Learner& L, const int32_t* rows, const int32_t* tgt, const float* w, int n) {
   const int R = L.R, M = L.M;
-  std::vector<int32_t> r(L.S, 0), t(L.S, 0);
-  std::vector<float> ww(L.S, 0.0f);
+  int32_t* r = reinterpret_cast<int32_t*>(L.pin);
+  int32_t* t = r + L.S;
+  float* ww = reinterpret_cast<float*>(t + L.S);
   for (int i = 0; i < n; ++i) {
     if (rows[i] < 0 || rows[i] >= R || (tgt && (tgt[i] < 0 || tgt[i] >= M)))
       throw Fail{HANDE_ERR_INVALID, "row or target orbital out of range"};
@@ -581,9 +590,22 @@ static void upload_batch(Engine& E, Learner& L, const int32_t* rows, const int32
     ww[i] = w ? w[i] : 1.0f;
     if (!(ww[i] >= 0.0f)) throw Fail{HANDE_ERR_INVALID, "sample weights must be >= 0"};
   }
-  CK(cudaMemcpyAsync(L.in_rows, r.data(), 4 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
-  CK(cudaMemcpyAsync(L.in_tgt, t.data(), 4 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
-  CK(cudaMemcpyAsync(L.in_w, ww.data(), 4 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
+  std::memset(r + n, 0, sizeof(int32_t) * (size_t)(L.S - n));
+  std::memset(t + n, 0, sizeof(int32_t) * (size_t)(L.S - n));
+  std::memset(ww + n, 0, sizeof(float) * (size_t)(L.S - n));
+  CK(cudaMemcpyAsync(L.in_rows, L.pin, 12 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
+}
+// the loss and the error word of the stream's work (synchronises)
+static double read_loss(Engine& E, Learner& L) {
+  char* p = L.pin + 12 * (size_t)L.S;
+  CK(cudaMemcpyAsync(p, L.loss, 16, cudaMemcpyDeviceToHost, E.stream));
+  CK(cudaStreamSynchronize(E.stream));
+  unsigned e;
+  std::memcpy(&e, p + 8, sizeof e);
+  if (e) throw Fail{HANDE_ERR_TIMEOUT, "a tensor-core GEMM wait timed out"};
+  double loss;
+  std::memcpy(&loss, p, sizeof loss);
+  return loss;
 }
 
 void learner_gradients(Engine& E, const int32_t* rows, const int32_t* tgt, const float* w, int n, float* grads,
@@ -594,12 +616,8 @@ void learner_gradients(Engine& E, const int32_t* rows, const int32_t* tgt, const
   CK(cudaMemsetAsync(L.err, 0, sizeof(unsigned), E.stream));
   backward(E, L, L.in_rows, L.in_tgt, L.in_w, E.stream);
   CK(cudaGetLastError());
-  unsigned e = 0;
   CK(cudaMemcpyAsync(grads, L.grad, sizeof(float) * L.nparam, cudaMemcpyDeviceToHost, E.stream));
-  CK(cudaMemcpyAsync(loss, L.loss, sizeof(double), cudaMemcpyDeviceToHost, E.stream));
-  CK(cudaMemcpyAsync(&e, L.err, sizeof e, cudaMemcpyDeviceToHost, E.stream));
-  CK(cudaStreamSynchronize(E.stream));
-  if (e) throw Fail{HANDE_ERR_TIMEOUT, "a tensor-core GEMM wait timed out"};
+  *loss = read_loss(E, L);
 }
 
 void learner_probabilities(Engine& E, const int32_t* rows, int n, float* probs) {
@@ -613,11 +631,8 @@ void learner_probabilities(Engine& E, const int32_t* rows, int n, float* probs) 
   k_lr_probs<<<(n * 32 + kLt - 1) / kLt, kLt, 0, E.stream>>>(L.Z3, L.param + L.ob3, L.in_rows, n, L.M, E.pmask_dev,
                                                               L.probs);
   CK(cudaGetLastError());
-  unsigned e = 0;
   CK(cudaMemcpyAsync(probs, L.probs, sizeof(float) * (size_t)n * L.M, cudaMemcpyDeviceToHost, E.stream));
-  CK(cudaMemcpyAsync(&e, L.err, sizeof e, cudaMemcpyDeviceToHost, E.stream));
-  CK(cudaStreamSynchronize(E.stream));
-  if (e) throw Fail{HANDE_ERR_TIMEOUT, "a tensor-core GEMM wait timed out"};
+  (void)read_loss(E, L);
 }
 
 void learner_refresh(Engine& E) {

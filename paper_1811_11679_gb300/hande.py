@@ -366,23 +366,31 @@ class Hande:
         memory: new arrays, or views of the given host_buffers(...) when they are
         large enough (page-locked buffers make the copies direct DMA)."""
         n = C.c_int64()
-        rc = self._lib.hande_get_walkers(self._h, None, None, None, None, 0, C.byref(n))
-        if rc not in (0, -3):
-            self._check(rc, "hande_get_walkers")
-        cap = n.value
-        if out is not None and len(out[1]) >= cap:
+
+        def fetch(keys, pops, hd, fl):
+            return self._lib.hande_get_walkers(self._h, keys.ctypes.data_as(C.POINTER(C.c_uint64)),
+                                               pops.ctypes.data_as(C.POINTER(C.c_int64)),
+                                               hd.ctypes.data_as(C.POINTER(C.c_double)),
+                                               fl.ctypes.data_as(C.POINTER(C.c_uint8)), len(pops), C.byref(n))
+
+        if out is not None and len(out[1]) > 0:   # one call when the list fits the given buffers
             keys, pops, hd, fl = out
-            cap = len(pops)
+            rc = fetch(*out)
+            if rc == 0:
+                m = n.value
+                return keys[:m], pops[:m], hd[:m], fl[:m]
+            if rc != -3 or n.value <= len(pops):
+                self._check(rc, "hande_get_walkers")
         else:
-            keys = np.zeros((cap, self.W), dtype=np.uint64)
-            pops = np.zeros(cap, dtype=np.int64)
-            hd = np.zeros(cap, dtype=np.float64)
-            fl = np.zeros(cap, dtype=np.uint8)
-        self._check(self._lib.hande_get_walkers(self._h, keys.ctypes.data_as(C.POINTER(C.c_uint64)),
-                                                pops.ctypes.data_as(C.POINTER(C.c_int64)),
-                                                hd.ctypes.data_as(C.POINTER(C.c_double)),
-                                                fl.ctypes.data_as(C.POINTER(C.c_uint8)), cap, C.byref(n)),
-                    "hande_get_walkers")
+            rc = self._lib.hande_get_walkers(self._h, None, None, None, None, 0, C.byref(n))
+            if rc not in (0, -3):
+                self._check(rc, "hande_get_walkers")
+        cap = n.value
+        keys = np.zeros((cap, self.W), dtype=np.uint64)
+        pops = np.zeros(cap, dtype=np.int64)
+        hd = np.zeros(cap, dtype=np.float64)
+        fl = np.zeros(cap, dtype=np.uint8)
+        self._check(fetch(keys, pops, hd, fl), "hande_get_walkers")
         m = n.value
         return keys[:m], pops[:m], hd[:m], fl[:m]
 
