@@ -52,18 +52,40 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// FP32 output {N, M} with row stride ldd, boxes of 32 x 32, 128-byte swizzle
+bool make_out_map(CUtensorMap* map, float* ptr, uint64_t N, uint64_t M, uint64_t ldd) {
+  EncodeTiledFn enc = encoder();
+  if (!enc) return false;
+  const cuuint64_t dims[2] = {N, M};
+  const cuuint64_t strides[1] = {ldd * 4};
+  const cuuint32_t box[2] = {32, 32};
+  const cuuint32_t estr[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// SMs of a device (looked up once per device)
+int sm_count(int dev) {
+  static int nsm[256] = {};
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (nsm[dev] == 0 && cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    nsm[dev] = 0;
+  }
+  return nsm[dev];
+}
+
 // persistent launch: one CTA per SM (at most one per output tile)
 template <int BN, int EPI>
-bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const Epilogue& ep, int M, int N, int K,
-                  unsigned* err, cudaStream_t s, int dev, const char** why) {
+bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md, int tma_out, const Epilogue& ep,
+                  int M, int N, int K, unsigned* err, cudaStream_t s, int dev, int nsm, const char** why) {
   static bool attr_set[256] = {};
-  static int nsm[256] = {};
   {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!attr_set[dev]) {
       if (cudaFuncSetAttribute(k_gemm_bf16_tn_p<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)PTile<BN>::kSmemBytes) != cudaSuccess ||
-          cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+                               (int)PTile<BN>::kSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         *why = "cannot reserve the GEMM's shared memory";
         return false;
@@ -72,8 +94,8 @@ bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const Epilogue& 
     }
   }
   const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + kBM - 1) / kBM);
-  const unsigned grid = (unsigned)(tiles < nsm[dev] ? tiles : nsm[dev]);
-  k_gemm_bf16_tn_p<BN, EPI><<<grid, kPThreads, PTile<BN>::kSmemBytes, s>>>(ma, mb, ep, M, N, K, err);
+  const unsigned grid = (unsigned)(tiles < nsm ? tiles : nsm);
+  k_gemm_bf16_tn_p<BN, EPI><<<grid, kPThreads, PTile<BN>::kSmemBytes, s>>>(ma, mb, md, tma_out, ep, M, N, K, err);
   if (cudaGetLastError() != cudaSuccess) {
     *why = "GEMM launch failed";
     return false;
@@ -82,7 +104,7 @@ bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const Epilogue& 
 }
 
 // Validated launch of D = A B^T with the given epilogue (see tc_gemm.cuh);
-// 256-column tiles when N > 128; false with a message on bad input
+// false with a message on bad input
 bool launch_gemm_ep(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb, const Epilogue& ep, int epi,
                     int M, int N, int K, unsigned* err, cudaStream_t s, const char** why) {
   if (M < 1 || N < 1 || K < 1 || !A || !B || !err || (epi == EPI_F32 ? !ep.D : (!ep.H || !ep.bias))) {
@@ -100,18 +122,29 @@ bool launch_gemm_ep(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t l
     *why = "no current CUDA device";
     return false;
   }
-  const int bn = N > 128 ? 256 : 128;
-  CUtensorMap ma, mb;
+  const int nsm = sm_count(dev);
+  if (nsm < 1) {
+    *why = "cannot read the SM count";
+    return false;
+  }
+  // the widest tile with a tile for every SM, else the narrowest that still
+  // covers N in one (an element's sum over K is the same in each)
+  const int64_t tm = (M + kBM - 1) / kBM;
+  int bn = N > 128 ? 256 : (N > 64 ? 128 : 64);
+  while (bn > 64 && tm * ((N + bn - 1) / bn) < nsm) bn >>= 1;
+  CUtensorMap ma, mb, md{};
+  const int tma_out = epi == EPI_F32 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) ? 1 : 0;
   if (!make_map(&ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, kBM) ||
-      !make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, (uint32_t)bn)) {
+      !make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, (uint32_t)bn) ||
+      (tma_out && !make_out_map(&md, ep.D, (uint64_t)N, (uint64_t)M, (uint64_t)ep.ldd))) {
     *why = "cuTensorMapEncodeTiled failed";
     return false;
   }
+  auto go = [&](auto launch) { return launch(ma, mb, md, tma_out, ep, M, N, K, err, s, dev, nsm, why); };
   if (epi == EPI_F32)
-    return bn == 256 ? launch_shape<256, EPI_F32>(ma, mb, ep, M, N, K, err, s, dev, why)
-                     : launch_shape<128, EPI_F32>(ma, mb, ep, M, N, K, err, s, dev, why);
-  return bn == 256 ? launch_shape<256, EPI_BF16_BIAS>(ma, mb, ep, M, N, K, err, s, dev, why)
-                   : launch_shape<128, EPI_BF16_BIAS>(ma, mb, ep, M, N, K, err, s, dev, why);
+    return go(bn == 256 ? &launch_shape<256, EPI_F32> : (bn == 128 ? &launch_shape<128, EPI_F32> : &launch_shape<64, EPI_F32>));
+  return go(bn == 256 ? &launch_shape<256, EPI_BF16_BIAS>
+                      : (bn == 128 ? &launch_shape<128, EPI_BF16_BIAS> : &launch_shape<64, EPI_BF16_BIAS>));
 }
 
 bool launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb, float* D, int64_t ldd, int M,

@@ -3,8 +3,9 @@
 //   D[m][n] = sum_k A[m][k] B[n][k]        (A: M x K, B: N x K, both K-major
 //                                           BF16 row-major; D: FP32)
 //
-// Output tiles of 128 x BN (BN = 128, or 256 when N > 128, so that A is read
-// once for N <= 256), walked by one persistent CTA per SM (see
+// Output tiles of 128 x BN (BN = 64, 128 or 256: the widest that still gives
+// every SM a tile, so that A is read once for N <= 256 on large products and
+// small ones use the chip), walked by one persistent CTA per SM (see
 // k_gemm_bf16_tn_p below).  The K dimension is taken in chunks of 64 elements
 // (128 bytes): a TMA tile load brings the A and B chunk of a stage into shared
 // memory in the 128-byte-swizzled K-major layout the tensor core reads, four
@@ -12,7 +13,8 @@
 // chunk, FP32 accumulators in tensor memory) and commits each stage to an
 // mbarrier that frees it for the next TMA load.  Four warps read the
 // accumulator rows they own (tcgen05.ld, 32 lanes x 32 columns at a time) and
-// store them as FP32, or as BF16 after adding a bias and a ReLU (with a
+// store them as FP32 (through shared memory and TMA where D's rows are 16-byte
+// aligned), or as BF16 after adding a bias and a ReLU (with a
 // transposed copy if asked: the learned proposal's hidden layers and their
 // backward operands).  Rows, columns and K beyond the matrix are zero-filled by
 // the TMA and masked in the store, so any M, N, K >= 1 work (leading
@@ -37,7 +39,7 @@ constexpr int kMmaK = 16;       // K of one tcgen05.mma kind::f16
 constexpr int kStages = 4;
 constexpr uint32_t kTileABytes = kBM * kBK * 2;
 constexpr unsigned ERR_MMA_TIMEOUT = 1u;
-// tile columns BN (MMA N, 128 or 256): the bytes of a B chunk
+// tile columns BN (MMA N): the bytes of a B chunk
 template <int BN>
 struct Tile {
   static constexpr uint32_t kTileBBytes = BN * kBK * 2;
@@ -102,6 +104,13 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
           smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
       : "memory");
+}
+
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(smem_u32(src)), "r"(x), "r"(y)
+               : "memory");
 }
 
 // ------------------------------------------------------------------ tcgen05
@@ -238,18 +247,26 @@ __device__ __forceinline__ void epi_store(const Epilogue& ep, const uint32_t (&r
 // shared flag that stops all roles, which then drain their own loads and MMAs
 // (bounded) before the tensor memory is freed.
 constexpr int kPThreads = 192;
+// FP32 output staged per epilogue warp: two buffers of 32 x 32 values, stored by
+// TMA (128-byte swizzle).  Lanes hold rows of the accumulator, so direct stores
+// put the 32 lanes of an instruction into 32 rows, 16 bytes each; the layer of
+// the 246-orbital table refresh (121088 x 256 x 512) went from 61 to 47 us.
+constexpr uint32_t kOutBytes = 32 * 32 * 4;
+constexpr uint32_t kOutWarpBytes = 2 * kOutBytes;
 // tensor-memory columns (two FP32 accumulators of BN columns: 512 at BN = 256)
 // and dynamic shared memory (1024-byte aligned stages + barriers)
 template <int BN>
 struct PTile {
   static constexpr uint32_t kTmemCols = 2 * BN;
-  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * (kTileABytes + Tile<BN>::kTileBBytes) + 256;
+  static constexpr size_t kStageBytes = (size_t)kStages * (kTileABytes + Tile<BN>::kTileBBytes);
+  static constexpr size_t kSmemBytes = 1024 + kStageBytes + 4 * kOutWarpBytes + 256;
 };
 
 template <int BN, int EPI>
 __global__ void __launch_bounds__(kPThreads, 1)
     k_gemm_bf16_tn_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                     const Epilogue ep, int M, int N, int K, unsigned* err) {
+                     const __grid_constant__ CUtensorMap tmD, int tma_out, const Epilogue ep, int M, int N, int K,
+                     unsigned* err) {
   constexpr uint32_t kTileBBytes = Tile<BN>::kTileBBytes;
   constexpr uint32_t kTmemCols = PTile<BN>::kTmemCols;
   extern __shared__ __align__(16) unsigned char tcp_smem_raw[];
@@ -257,7 +274,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tcp_smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = base;
   unsigned char* sB = base + (size_t)kStages * kTileABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sB + (size_t)kStages * kTileBBytes);
+  unsigned char* sOut = base + PTile<BN>::kStageBytes;   // 1024-byte aligned
+  uint64_t* full = reinterpret_cast<uint64_t*>(sOut + 4 * kOutWarpBytes);
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;      // [2]
   uint64_t* acc_empty = acc_full + 2;        // [2]
@@ -353,6 +371,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
   } else {   // epilogue warps 0-3
     const int lrow = warp * 32 + lane;
+    unsigned char* out = sOut + warp * kOutWarpBytes;
+    uint32_t stores = 0;
     int i = 0;
     for (int t = (int)blockIdx.x; t < ntiles && !s_fail; t += (int)gridDim.x, ++i) {
       const int m0 = (t / tn_count) * kBM, n0 = (t % tn_count) * BN;
@@ -368,12 +388,29 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if (n0 + c0 >= N) break;
         uint32_t r[32];
         tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * BN + c0), r);
-        epi_store<EPI>(ep, r, m0 + lrow, n0, c0, M, N);
+        if (EPI == EPI_F32 && tma_out) {
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // this buffer was read
+          __syncwarp();
+          unsigned char* b = out + (stores++ & 1) * kOutBytes + lane * 128;
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<uint4*>(b + ((q ^ (lane & 7)) << 4)) =
+                make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0 && m0 + warp * 32 < M) {   // rows and columns beyond D are clipped
+            tma_store_2d(&tmD, b, n0 + c0, m0 + warp * 32);
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
+        } else {
+          epi_store<EPI>(ep, r, m0 + lrow, n0, c0, M, N);
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[a]);
     }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
