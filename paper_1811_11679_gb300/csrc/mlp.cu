@@ -133,7 +133,8 @@ bool launch_gemm_ep(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t l
   int bn = N > 128 ? 256 : (N > 64 ? 128 : 64);
   while (bn > 64 && tm * ((N + bn - 1) / bn) < nsm) bn >>= 1;
   CUtensorMap ma, mb, md{};
-  const int tma_out = epi == EPI_F32 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) ? 1 : 0;
+  // (a TMA store clips a row in 16-byte steps, so N is a multiple of 4 too)
+  const int tma_out = epi == EPI_F32 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) && !(N & 3) ? 1 : 0;
   if (!make_map(&ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, kBM) ||
       !make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, (uint32_t)bn) ||
       (tma_out && !make_out_map(&md, ep.D, (uint64_t)N, (uint64_t)M, (uint64_t)ep.ldd))) {
