@@ -62,6 +62,12 @@ struct Ops {
   size_t attempt_smem;
 };
 
+// iterations in one graph launch while nothing on the host is due between them
+// (even: the list is back in its buffer).  A launch per iteration left 2-4 us
+// between iterations of 40-170 us.  Programmatic dependent launches between the
+// kernels were measured beside it and left out: they gained nothing on top and
+// cost the long iterations 3%.
+constexpr int kGraphIters = 4;
 constexpr int kPinRecords = 64;   // records read back through the page-locked block
 constexpr int kPhases = 10;   // timed phases of one iteration
 
@@ -89,7 +95,9 @@ struct Engine {
   int merge_warp_grid = 0;
   size_t merge_smem_bytes = 0;
   int attempt_grid = 0;
+  // captured iterations by list buffer and core state: one, and kGraphIters in a row
   cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+  cudaGraphExec_t graph_n[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   int cur = 0;
   int64_t host_iter = 0;
   int64_t epoch = 0;   // incremented whenever the parameter block changes (graphs dropped)
@@ -138,6 +146,7 @@ void learner_probabilities(Engine& E, const int32_t* rows, int n, float* probs);
 void learner_refresh(Engine& E);
 void learner_step(Engine& E);
 bool learner_due(const Engine& E);
+int learner_period(const Engine& E);   // 0: no online training
 // batches (host.cu)
 bool engine_batchable(const Engine& E);
 bool engine_after_iteration(Engine& E);

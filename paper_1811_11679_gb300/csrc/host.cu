@@ -26,10 +26,11 @@ void release_all(Engine& E) {
   learner_release(E);
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b)
-      if (E.graph[a][b]) {
-        cudaGraphExecDestroy(E.graph[a][b]);
-        E.graph[a][b] = nullptr;
-      }
+      for (cudaGraphExec_t* g : {&E.graph[a][b], &E.graph_n[a][b]})
+        if (*g) {
+          cudaGraphExecDestroy(*g);
+          *g = nullptr;
+        }
   cudaStreamSynchronize(E.stream);
   for (auto& blk : E.blocks) {
     if (E.has_alloc) E.alloc.free(blk.first, blk.second, E.alloc.user);
@@ -489,11 +490,14 @@ void tau_search_step(Engine& E) {
   }
 }
 
-void ensure_graph(Engine& E, int cur, int core) {
-  if (E.graph[cur][core]) return;
+// the captured graph of `iters` (1 or kGraphIters) iterations starting in list
+// buffer cur
+void ensure_graph(Engine& E, int cur, int core, int iters) {
+  cudaGraphExec_t& slot = iters == 1 ? E.graph[cur][core] : E.graph_n[cur][core];
+  if (slot) return;
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(E.cap_stream, cudaStreamCaptureModeThreadLocal));
-  E.ops.iteration(E, cur, core != 0, E.cap_stream, nullptr);
+  for (int i = 0; i < iters; ++i) E.ops.iteration(E, cur ^ (i & 1), core != 0, E.cap_stream, nullptr);
   cudaError_t launch_err = cudaGetLastError();
   CK(cudaStreamEndCapture(E.cap_stream, &g));
   if (launch_err != cudaSuccess) {
@@ -504,16 +508,17 @@ void ensure_graph(Engine& E, int cur, int core) {
   cudaError_t ie = cudaGraphInstantiate(&ex, g, 0);
   cudaGraphDestroy(g);
   CK(ie);
-  E.graph[cur][core] = ex;
+  slot = ex;
 }
 
 void drop_graphs(Engine& E, int core) {
   E.epoch += 1;   // the parameter block may have changed: batch graphs are rebuilt too
   for (int c = 0; c < 2; ++c)
-    if (E.graph[c][core]) {
-      cudaGraphExecDestroy(E.graph[c][core]);
-      E.graph[c][core] = nullptr;
-    }
+    for (cudaGraphExec_t* g : {&E.graph[c][core], &E.graph_n[c][core]})
+      if (*g) {
+        cudaGraphExecDestroy(*g);
+        *g = nullptr;
+      }
 }
 
 // run the int64 scan machinery on natt[0..ndet[cur]) -> att_begin, total -> scan_total
@@ -1040,7 +1045,17 @@ hande_status hande_iterate(hande_ctx* ctx, int n) {
   return run_guarded(&E, [&]() -> hande_status {
     for (int k = 0; k < n; ++k) {
       int core = E.core_active ? 1 : 0;
-      ensure_graph(E, E.cur, core);
+      // several iterations per launch when no host work is due between them
+      const bool core_due = E.core_size > 0 && !E.core_active && E.core_start > E.host_iter &&
+                            E.core_start <= E.host_iter + kGraphIters;
+      if (n - k >= kGraphIters && !(E.learn && learner_period(E) > 0) && !E.tau_searching && !core_due) {
+        ensure_graph(E, E.cur, core, kGraphIters);
+        CK(cudaGraphLaunch(E.graph_n[E.cur][core], E.stream));
+        E.host_iter += kGraphIters;
+        k += kGraphIters - 1;
+        continue;
+      }
+      ensure_graph(E, E.cur, core, 1);
       CK(cudaGraphLaunch(E.graph[E.cur][core], E.stream));
       E.cur ^= 1;
       E.host_iter += 1;
@@ -1472,6 +1487,8 @@ hande_status hande_autotune(hande_ctx* ctx, int iterations, hande_tuning* out) {
           drop_graphs(E, 0);
           drop_graphs(E, 1);
           hande_status st = hande_iterate(ctx, 1);   // captures the graphs for this shape
+          if (st == HANDE_OK && iterations >= kGraphIters)
+            for (int c = 0; c < 2; ++c) ensure_graph(E, c, E.core_active ? 1 : 0, kGraphIters);
           if (st == HANDE_OK) {
             CK(cudaEventRecord(e0, E.stream));
             st = hande_iterate(ctx, iterations);

@@ -671,6 +671,8 @@ void learner_step(Engine& E) {
   CK(cudaGraphLaunch(L.graph, E.stream));
 }
 
+int learner_period(const Engine& E) { return E.learn ? E.learn->period : 0; }
+
 bool learner_due(const Engine& E) {
   return E.learn && E.learn->period > 0 && E.host_iter % E.learn->period == 0;
 }
