@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -54,7 +55,7 @@ struct Learner {
   uint16_t *X = nullptr, *XT = nullptr, *Xtab = nullptr;
   uint16_t *H1 = nullptr, *H2 = nullptr, *H1T = nullptr, *H2T = nullptr;
   uint16_t *G3 = nullptr, *G3T = nullptr, *dZ2 = nullptr, *dZ2T = nullptr, *dZ1 = nullptr, *dZ1T = nullptr;
-  float *Z3 = nullptr, *dH = nullptr;
+  float *Z3 = nullptr, *dH = nullptr, *ws = nullptr;   // ws: parts of a weight gradient
   float* wsum = nullptr;
   double* loss = nullptr;
   unsigned* err = nullptr;   // the word behind the loss
@@ -69,37 +70,74 @@ struct Learner {
 namespace {
 
 constexpr int kLt = 256;
+constexpr int kMaxParts = 16;   // parts of a weight gradient's sum over the samples
 
 __device__ __forceinline__ uint16_t f2bf(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float bf2f(uint16_t b) { return __bfloat162float(__ushort_as_bfloat16(b)); }
 
 // features x(r) of rows[0 .. S) (rows with w == 0, or beyond count, are zero):
-// X [S][kin] and, if XT, its transpose [kin][S]
-__global__ void k_lr_features(const int32_t* rows, const float* w, int count, int S, int M, int kin, uint16_t* X,
-                              uint16_t* XT) {
-  const int64_t total = (int64_t)S * kin;
+// X [S][kin] and, if XT, its transpose [kin][S]; eight values per thread and
+// store, along a row of X or of XT (S and kin are multiples of 64).  One value
+// per thread with a 2-byte transposed store took 8-9 us for 4096 rows, this
+// 4.
+__global__ void __launch_bounds__(kLt) k_lr_features(const int32_t* rows, const float* w, int count, int S, int M,
+                                                     int kin, uint16_t* X, uint16_t* XT) {
+  const int64_t half = (int64_t)S * kin / 8, total = XT ? 2 * half : half;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(i / kin), k = (int)(i % kin);
-    uint16_t v = 0;
-    if (n < count && (!w || w[n] > 0.0f)) {
-      const int r = rows[n], same = r & 1, IJ = r >> 1, I = IJ / M, J = IJ % M;
-      if (k == I || k == M + J || (k == 2 * M && same)) v = 0x3F80;   // BF16 1.0
+    uint32_t v[4] = {0u, 0u, 0u, 0u};
+    if (i < half) {             // X[n][k0 ..]
+      const int n = (int)(i / (kin / 8)), k0 = (int)(i % (kin / 8)) * 8;
+      const bool on = n < count && (!w || w[n] > 0.0f);
+      const int r = on ? rows[n] : 0, same = r & 1, IJ = r >> 1, I = IJ / M, J = M + IJ % M;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = k0 + u;
+        if (on && (k == I || k == J || (k == 2 * M && same))) v[u / 2] |= 0x3F80u << (16 * (u & 1));   // BF16 1.0
+      }
+      reinterpret_cast<uint4*>(X)[i] = make_uint4(v[0], v[1], v[2], v[3]);
+    } else {                    // XT[k][n0 ..]
+      const int64_t e = i - half;
+      const int k = (int)(e / (S / 8)), n0 = (int)(e % (S / 8)) * 8;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int n = n0 + u;
+        const bool on = n < count && (!w || w[n] > 0.0f);
+        const int r = on ? rows[n] : 0, same = r & 1, IJ = r >> 1;
+        if (on && (k < M ? k == IJ / M : (k < 2 * M ? k - M == IJ % M : (k == 2 * M && same))))
+          v[u / 2] |= 0x3F80u << (16 * (u & 1));
+      }
+      reinterpret_cast<uint4*>(XT)[e] = make_uint4(v[0], v[1], v[2], v[3]);
     }
-    X[i] = v;
-    if (XT) XT[(int64_t)k * S + n] = v;
   }
 }
 
 // dZ = (h > 0) ? dH : 0 in BF16 [n][Hd] and transposed [Hd][ldT], h the layer's
-// BF16 ReLU output (positive exactly where the pre-activation is)
-__global__ void k_lr_relu_back(const float* dH, const uint16_t* Hact, int n, int Hd, uint16_t* dZ, uint16_t* dZT,
-                               int ldT) {
-  const int64_t total = (int64_t)n * Hd;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / Hd), j = (int)(i % Hd);
-    const uint16_t g = (Hact[i] != 0 && !(Hact[i] & 0x8000)) ? f2bf(dH[i]) : (uint16_t)0;
-    dZ[i] = g;
-    dZT[(int64_t)j * ldT + r] = g;
+// BF16 ReLU output (positive exactly where the pre-activation is); one block per
+// 64 x 64 tile, transposed through shared memory (n and Hd are multiples of 64).
+// Transposed 2-byte stores from global order took 12 us for 4096 x 256, this
+// 6.5.
+constexpr int kRt = 64;
+__global__ void __launch_bounds__(kLt) k_lr_relu_back(const float* dH, const uint16_t* Hact, int Hd, uint16_t* dZ,
+                                                      uint16_t* dZT, int ldT) {
+  __shared__ uint16_t tile[kRt][kRt + 2];
+  const int r0 = (int)blockIdx.x * kRt, j0 = (int)blockIdx.y * kRt;
+  for (int e = threadIdx.x; e < kRt * kRt / 2; e += blockDim.x) {   // two columns per thread
+    const int r = e / (kRt / 2), j = e % (kRt / 2) * 2;
+    const int64_t at = (int64_t)(r0 + r) * Hd + j0 + j;
+    const float2 g = *reinterpret_cast<const float2*>(dH + at);
+    const uint32_t h = *reinterpret_cast<const uint32_t*>(Hact + at);
+    const uint16_t h0 = (uint16_t)h, h1 = (uint16_t)(h >> 16);
+    const uint16_t g0 = h0 != 0 && !(h0 & 0x8000) ? f2bf(g.x) : (uint16_t)0;
+    const uint16_t g1 = h1 != 0 && !(h1 & 0x8000) ? f2bf(g.y) : (uint16_t)0;
+    *reinterpret_cast<uint32_t*>(dZ + at) = (uint32_t)g0 | ((uint32_t)g1 << 16);
+    tile[r][j] = g0;
+    tile[r][j + 1] = g1;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < kRt * kRt / 2; e += blockDim.x) {   // two rows per thread
+    const int j = e / (kRt / 2), r = e % (kRt / 2) * 2;
+    *reinterpret_cast<uint32_t*>(dZT + (int64_t)(j0 + j) * ldT + r0 + r) =
+        (uint32_t)tile[r][j] | ((uint32_t)tile[r + 1][j] << 16);
   }
 }
 
@@ -304,10 +342,36 @@ inline int grid_for(int64_t n) {
   return g < 1 ? 1 : (int)g;
 }
 
+// D[i][j] = sum over the parts of ws[part][i][j], in order
+__global__ void __launch_bounds__(kLt) k_lr_sum_parts(const float* ws, int parts, int64_t n, int64_t stride, float* D) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    float s = 0.0f;
+    for (int p = 0; p < parts; ++p) s += ws[p * stride + i];
+    D[i] = s;
+  }
+}
+
 void gemm(Learner& L, const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb, float* D, int64_t ldd, int m,
           int n, int k, cudaStream_t s) {
   const char* why = "";
   if (!tc::launch_gemm(A, lda, B, ldb, D, ldd, m, n, k, L.err, s, &why)) throw Fail{HANDE_ERR_CUDA, why};
+}
+
+// a weight gradient D [m][n] = A B^T over the samples (k = S): few output tiles
+// and a long sum, so the sum is divided among the SMs and the parts added after
+// (one tile's 64 chunks in a row took 19 us on at most 8 SMs)
+void gemm_long(Learner& L, const uint16_t* A, const uint16_t* B, float* D, int m, int n, cudaStream_t s) {
+  const int chunks = (L.S + tc::kBK - 1) / tc::kBK, per = (chunks + kMaxParts - 1) / kMaxParts;
+  const int parts = (chunks + per - 1) / per;
+  tc::Epilogue ep{};
+  ep.D = L.ws;
+  ep.ldd = n;
+  ep.parts = parts;
+  ep.part_chunks = per;
+  ep.part_stride = (int64_t)m * n;
+  const char* why = "";
+  if (!tc::launch_gemm_ep(A, L.S, B, L.S, ep, tc::EPI_F32, m, n, L.S, L.err, s, &why)) throw Fail{HANDE_ERR_CUDA, why};
+  k_lr_sum_parts<<<grid_for((int64_t)m * n), kLt, 0, s>>>(L.ws, parts, (int64_t)m * n, (int64_t)m * n, D);
 }
 
 // forward of `nrows` feature rows X [nrows][kin] to the logits Z3 [nrows][M]
@@ -339,22 +403,22 @@ void forward(Learner& L, const uint16_t* X, int nrows, bool train, cudaStream_t 
 void backward(Engine& E, Learner& L, const int32_t* rows, const int32_t* tgt, const float* w, cudaStream_t s) {
   const int H = L.H, S = L.S, M = L.M;
   k_lr_wsum<<<1, kLt, 0, s>>>(w, S, L.wsum);
-  k_lr_features<<<grid_for((int64_t)S * L.kin), kLt, 0, s>>>(rows, w, S, S, M, L.kin, L.X, L.XT);
+  k_lr_features<<<grid_for((int64_t)S * L.kin / 4), kLt, 0, s>>>(rows, w, S, S, M, L.kin, L.X, L.XT);
   forward(L, L.X, S, true, s);
   CK(cudaMemsetAsync(L.loss, 0, sizeof(double), s));
   k_lr_softmax_grad<<<(S * 32 + kLt - 1) / kLt, kLt, 0, s>>>(L.Z3, L.param + L.ob3, rows, tgt, w, L.wsum, S, M, L.M8,
                                                               E.pmask_dev, L.G3, L.G3T, L.loss);
   float* g = L.grad;
-  gemm(L, L.G3T, S, L.H2T, S, g + L.oW3, H, M, H, S, s);                 // dW3 = G3^T H2
+  gemm_long(L, L.G3T, L.H2T, g + L.oW3, M, H, s);                         // dW3 = G3^T H2
   k_lr_colsum<<<M, kLt, 0, s>>>(L.G3T, S, g + L.ob3);
   gemm(L, L.G3, L.M8, L.W3bT, L.M8, L.dH, H, S, H, M, s);                // dH2 = G3 W3
-  k_lr_relu_back<<<grid_for((int64_t)S * H), kLt, 0, s>>>(L.dH, L.H2, S, H, L.dZ2, L.dZ2T, S);
+  k_lr_relu_back<<<dim3(S / kRt, H / kRt), kLt, 0, s>>>(L.dH, L.H2, H, L.dZ2, L.dZ2T, S);
   k_lr_colsum<<<H, kLt, 0, s>>>(L.dZ2T, S, g + L.ob2);
-  gemm(L, L.dZ2T, S, L.H1T, S, g + L.oW2, H, H, H, S, s);                // dW2 = dZ2^T H1
+  gemm_long(L, L.dZ2T, L.H1T, g + L.oW2, H, H, s);                        // dW2 = dZ2^T H1
   gemm(L, L.dZ2, H, L.W2bT, H, L.dH, H, S, H, H, s);                     // dH1 = dZ2 W2
-  k_lr_relu_back<<<grid_for((int64_t)S * H), kLt, 0, s>>>(L.dH, L.H1, S, H, L.dZ1, L.dZ1T, S);
+  k_lr_relu_back<<<dim3(S / kRt, H / kRt), kLt, 0, s>>>(L.dH, L.H1, H, L.dZ1, L.dZ1T, S);
   k_lr_colsum<<<H, kLt, 0, s>>>(L.dZ1T, S, g + L.ob1);
-  gemm(L, L.dZ1T, S, L.XT, S, g + L.oW1, L.din, H, L.din, S, s);         // dW1 = dZ1^T X
+  gemm_long(L, L.dZ1T, L.XT, g + L.oW1, H, L.din, s);                     // dW1 = dZ1^T X
 }
 
 void to_bf16(Learner& L, cudaStream_t s) {
@@ -504,6 +568,7 @@ void learner_attach(Engine& E, const hande_learning& in) {
   L.dZ1T = dalloc<uint16_t>(E, (size_t)H * L.S);
   L.Z3 = dalloc<float>(E, (size_t)L.rows_cap * M);
   L.dH = dalloc<float>(E, (size_t)L.S * H);
+  L.ws = dalloc<float>(E, (size_t)kMaxParts * H * std::max(std::max(H, L.din), M));
   L.wsum = dalloc<float>(E, 1);
   L.loss = dalloc<double>(E, 2);
   L.err = reinterpret_cast<unsigned*>(L.loss + 1);
@@ -530,7 +595,7 @@ void learner_attach(Engine& E, const hande_learning& in) {
   for (int i = 0; i < L.Rp; ++i) rows[i] = i < L.R ? i : 0;
   int32_t* drows = dalloc<int32_t>(E, L.Rp);
   CK(cudaMemcpyAsync(drows, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice, s));
-  k_lr_features<<<grid_for((int64_t)L.Rp * L.kin), kLt, 0, s>>>(drows, nullptr, L.R, L.Rp, M, L.kin, L.Xtab, nullptr);
+  k_lr_features<<<grid_for((int64_t)L.Rp * L.kin / 8), kLt, 0, s>>>(drows, nullptr, L.R, L.Rp, M, L.kin, L.Xtab, nullptr);
   CK(cudaGetLastError());
   // seeded initial weights: uniform in +-sqrt(6 / fan_in), zero biases
   std::vector<float> p((size_t)L.nparam, 0.0f);
@@ -625,7 +690,7 @@ void learner_probabilities(Engine& E, const int32_t* rows, int n, float* probs) 
   if (n < 1 || n > L.S) throw Fail{HANDE_ERR_INVALID, "row count must be in [1, batch]"};
   upload_batch(E, L, rows, nullptr, nullptr, n);
   CK(cudaMemsetAsync(L.err, 0, sizeof(unsigned), E.stream));
-  k_lr_features<<<grid_for((int64_t)L.S * L.kin), kLt, 0, E.stream>>>(L.in_rows, nullptr, n, L.S, L.M, L.kin, L.X,
+  k_lr_features<<<grid_for((int64_t)L.S * L.kin / 8), kLt, 0, E.stream>>>(L.in_rows, nullptr, n, L.S, L.M, L.kin, L.X,
                                                                        nullptr);
   forward(L, L.X, L.S, false, E.stream);
   k_lr_probs<<<(n * 32 + kLt - 1) / kLt, kLt, 0, E.stream>>>(L.Z3, L.param + L.ob3, L.in_rows, n, L.M, E.pmask_dev,

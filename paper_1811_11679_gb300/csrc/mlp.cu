@@ -93,7 +93,7 @@ bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMa
       attr_set[dev] = true;
     }
   }
-  const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + kBM - 1) / kBM);
+  const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + kBM - 1) / kBM) * (ep.parts > 1 ? ep.parts : 1);
   const unsigned grid = (unsigned)(tiles < nsm ? tiles : nsm);
   k_gemm_bf16_tn_p<BN, EPI><<<grid, kPThreads, PTile<BN>::kSmemBytes, s>>>(ma, mb, md, tma_out, ep, M, N, K, err);
   if (cudaGetLastError() != cudaSuccess) {
@@ -131,10 +131,10 @@ bool launch_gemm_ep(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t l
   // covers N in one (an element's sum over K is the same in each)
   const int64_t tm = (M + kBM - 1) / kBM;
   int bn = N > 128 ? 256 : (N > 64 ? 128 : 64);
-  while (bn > 64 && tm * ((N + bn - 1) / bn) < nsm) bn >>= 1;
+  while (bn > 64 && tm * ((N + bn - 1) / bn) * (ep.parts > 1 ? ep.parts : 1) < nsm) bn >>= 1;
   CUtensorMap ma, mb, md{};
   // (a TMA store clips a row in 16-byte steps, so N is a multiple of 4 too)
-  const int tma_out = epi == EPI_F32 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) && !(N & 3) ? 1 : 0;
+  const int tma_out = epi == EPI_F32 && ep.parts <= 1 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) && !(N & 3) ? 1 : 0;
   if (!make_map(&ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, kBM) ||
       !make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, (uint32_t)bn) ||
       (tma_out && !make_out_map(&md, ep.D, (uint64_t)N, (uint64_t)M, (uint64_t)ep.ldd))) {

@@ -50,6 +50,9 @@ enum { EPI_F32 = 0, EPI_BF16_BIAS = 1 };
 struct Epilogue {
   float* D;                 // EPI_F32: D[row * ldd + col]
   int64_t ldd;
+  int parts;                // EPI_F32: K divided into this many parts (0, 1: one) of part_chunks
+  int part_chunks;          //   64-element chunks, part p stored at D + p part_stride
+  int64_t part_stride;
   uint16_t* H;              // EPI_BF16_BIAS: H[row * ldh + col] = bf16(act(D + bias[col]))
   int64_t ldh;
   uint16_t* HT;             //   and, if not null, HT[col * ldt + row]
@@ -286,7 +289,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
   const int nk = (K + kBK - 1) / kBK;
   const int tn_count = (N + BN - 1) / BN, tm_count = (M + kBM - 1) / kBM;
-  const int ntiles = tn_count * tm_count;
+  const int parts = ep.parts > 1 ? ep.parts : 1, per = parts > 1 ? ep.part_chunks : nk;
+  const int nout = tn_count * tm_count, ntiles = nout * parts;   // work items: part-major
 
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -317,8 +321,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
       int64_t fill = 0;   // chunk loads issued over all tiles
       int64_t landed = 0;
       for (int t = (int)blockIdx.x; t < ntiles && !s_fail; t += (int)gridDim.x) {
-        const int m0 = (t / tn_count) * kBM, n0 = (t % tn_count) * BN;
-        for (int kc = 0; kc < nk && !s_fail; ++kc, ++fill) {
+        const int o = t % nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
+        const int k0 = t / nout * per, k1 = k0 + per < nk ? k0 + per : nk;
+        for (int kc = k0; kc < k1 && !s_fail; ++kc, ++fill) {
           const int st = (int)(fill % kStages);
           const uint32_t ph = (uint32_t)((fill / kStages) & 1);
           if (!mbar_wait(&empty[st], ph ^ 1u)) {
@@ -348,7 +353,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
         }
         tc_fence_after();
         const uint32_t dcol = tmem + (uint32_t)(a * BN);
-        for (int kc = 0; kc < nk; ++kc, ++use) {
+        const int k0 = t / nout * per, k1 = k0 + per < nk ? k0 + per : nk;
+        for (int kc = k0; kc < k1; ++kc, ++use) {
           const int st = (int)(use % kStages);
           if (!mbar_wait(&full[st], (uint32_t)((use / kStages) & 1))) {
             fail();
@@ -360,7 +366,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
 #pragma unroll
           for (int j = 0; j < kBK / kMmaK; ++j)
             tc_mma(dcol, sw128_kmajor_desc(a0 + 32u * j), sw128_kmajor_desc(b0 + 32u * j), idesc,
-                   (kc > 0 || j > 0) ? 1u : 0u);
+                   (kc > k0 || j > 0) ? 1u : 0u);
           tc_commit(&empty[st]);
         }
         if (s_fail) break;
@@ -375,7 +381,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
     uint32_t stores = 0;
     int i = 0;
     for (int t = (int)blockIdx.x; t < ntiles && !s_fail; t += (int)gridDim.x, ++i) {
-      const int m0 = (t / tn_count) * kBM, n0 = (t % tn_count) * BN;
+      const int o = t % nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
+      Epilogue pe = ep;
+      pe.D += (int64_t)(t / nout) * ep.part_stride;
       const int a = i & 1;
       const bool ok = mbar_wait(&acc_full[a], (uint32_t)((i >> 1) & 1));
       if (!__all_sync(0xffffffffu, ok)) {   // warp-uniform (the accumulator reads are warp-collective)
@@ -403,7 +411,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
         } else {
-          epi_store<EPI>(ep, r, m0 + lrow, n0, c0, M, N);
+          epi_store<EPI>(pe, r, m0 + lrow, n0, c0, M, N);
         }
       }
       tc_fence_before();
