@@ -142,24 +142,33 @@ __global__ void __launch_bounds__(kLt) k_lr_relu_back(const float* dH, const uin
   }
 }
 
-// *wsum = sum of the sample weights (one block, fixed order; n a multiple of 4)
-constexpr int kWs = 1024;
-__global__ void __launch_bounds__(kWs) k_lr_wsum(const float* w, int n, float* wsum) {
-  __shared__ float sh[kWs / 32];
+// *wsum = sum of the sample weights (one block, fixed order: each thread's
+// strided elements, then halves onto halves; n a multiple of 128).  The order is
+// kept because a last-bit change of the sum moves BF16 roundings of every
+// sample's gradient; eight loads are in flight ahead of the ordered additions.
+__global__ void __launch_bounds__(kLt) k_lr_wsum(const float* w, int n, float* wsum) {
+  __shared__ float sh[kLt];
+  const int t = (int)threadIdx.x;
   float s = 0.0f;
-  for (int i = threadIdx.x; i < n / 4; i += blockDim.x) {
-    const float4 v = reinterpret_cast<const float4*>(w)[i];
-    s += (v.x + v.y) + (v.z + v.w);
+  for (int i0 = t; i0 < n; i0 += 8 * kLt) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i0 + u * kLt < n ? w[i0 + u * kLt] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  sh[t] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    s = sh[threadIdx.x];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) *wsum = s;
+  for (int o = kLt / 2; o >= 32; o >>= 1) {
+    if (t < o) sh[t] += sh[t + o];
+    __syncthreads();
+  }
+  if (t < 32) {
+    s = sh[t];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (t == 0) *wsum = s;
   }
 }
 
@@ -425,7 +434,7 @@ void forward(Learner& L, const uint16_t* X, int nrows, bool train, cudaStream_t 
 // gradients of the loss of the batch (rows, tgt, w) [S] into L.grad and L.loss
 void backward(Engine& E, Learner& L, const int32_t* rows, const int32_t* tgt, const float* w, cudaStream_t s) {
   const int H = L.H, S = L.S, M = L.M;
-  k_lr_wsum<<<1, kWs, 0, s>>>(w, S, L.wsum);
+  k_lr_wsum<<<1, kLt, 0, s>>>(w, S, L.wsum);
   k_lr_features<<<grid_for((int64_t)S * L.kin / 4), kLt, 0, s>>>(rows, w, S, S, M, L.kin, L.X, L.XT);
   forward(L, L.X, S, true, s);
   CK(cudaMemsetAsync(L.loss, 0, sizeof(double), s));
