@@ -928,7 +928,7 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     P.natt = dalloc<int64_t>(E, cap);
     P.att_begin = dalloc<int64_t>(E, cap);
     P.part = dalloc<int64_t>(E, kScanBlocks + 1);
-    const size_t det_states = (size_t)(list_tiles(cap) + 16);   // a short list has up to 16 smaller tiles
+    const size_t det_states = (size_t)(cap / kDetTile + 33);   // a short list has up to 32 smaller tiles
     P.det_state = dalloc<unsigned long long>(E, det_states);
     CK(cudaMemsetAsync(P.det_state, 0, det_states * sizeof(unsigned long long), E.stream));
     P.s_key = dalloc<uint64_t>(E, (size_t)scap * E.W);

@@ -413,19 +413,23 @@ __device__ __forceinline__ unsigned long long lookback_warp(DevState* st, unsign
 }
 
 // One pass over the list: estimators, initiator flags, death, attempt counts and
-// their exclusive scan (att_begin), in tiles of 1024 entries taken in ticket
+// their exclusive scan (att_begin), in tiles of 512 entries taken in ticket
 // order (smaller ones for a short list, so that its FP64 work spreads over the
 // SMs).  The scan is chained through the tiles (look-back) instead of a second
 // and third kernel over the counts: those cost 21 us of a 930 us iteration on
 // 2.3e6 determinants, and two launches of the 17 of a small one.  Entries
 // connected to the reference (a percent of a large list) are queued and their
 // matrix elements evaluated by full warps while warp 0 looks back.
-// Bound: the FP64 unit (death: five operations per entry) and Philox issue.
-constexpr int kDetThreads = 512;
+// Bound: Philox issue and the FP64 unit (death: five operations per entry) at half
+// occupancy.  Four blocks of 256 threads per SM instead of two of 512, so that
+// others run while one waits at its look-back: one pass of ueg 14e/38 3293 ->
+// 3231 us, proposal table 1821 -> 1783, hubbard 2d 18 4984 -> 4902, molecule 1e7
+// 14184 -> 14053.
+constexpr int kDetThreads = 256;
 constexpr int kDetItems = 2;
-constexpr int kDetTile = kDetThreads * kDetItems;   // 1024
+constexpr int kDetTile = kDetThreads * kDetItems;   // 512
 constexpr int kDetWarps = kDetThreads / 32;
-static_assert(kDetItems * kDetWarps == 32, "one warp scans the tile's warp sums");
+static_assert(kDetItems * kDetWarps <= 32, "one warp scans the tile's warp sums");
 
 template <int W, int SYS>
 __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid vg) {
@@ -441,10 +445,11 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
   const int64_t t = st->iter + 1;
   const double S = st->shift;
   // short lists in smaller tiles, down to 64 entries, as long as that makes at
-  // most 16 tiles, each with a block of its own (Hubbard ring: 10.7 -> 6.6 us;
-  // with up to 512 tiles lists of 1e5 entries took longer, 12 -> 17 us)
+  // most 32 tiles (one look-back step), each with a block of its own (Hubbard
+  // ring: 10.7 -> 6.6 us; with up to 512 tiles lists of 1e5 entries took longer,
+  // 12 -> 17 us)
   int64_t size = kDetTile;
-  while (size > 64 && n <= size / 2 * (vg.n < 16 ? vg.n : 16)) size >>= 1;
+  while (size > 64 && n <= size / 2 * (vg.n < 32 ? vg.n : 32)) size >>= 1;
   const int64_t tiles = (n + size - 1) / size;
   if (__syncthreads_or((int)st->error) || vg.b >= tiles) return;   // no tile for this block
   const Key<W> d0 = ref_key<W>(P);
@@ -559,7 +564,7 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
     }
     __syncthreads();
     if (wid == 0) {
-      const unsigned long long v = wpre[lane];
+      const unsigned long long v = lane < kDetItems * kDetWarps ? wpre[lane] : 0ull;
       unsigned long long x = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -593,10 +598,10 @@ __device__ __forceinline__ void d_det_pass(const Params& P, int cur, const VGrid
   if (threadIdx.x == 0 && (c.lo | (uint64_t)c.hi)) atomic_add_i128(st->num, c);
 }
 template <int W, int SYS>
-__global__ void __launch_bounds__(kDetThreads, W == 8 ? 1 : 2) k_det_pass(Params P, int cur) { d_det_pass<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+__global__ void __launch_bounds__(kDetThreads, W == 8 ? 2 : 4) k_det_pass(Params P, int cur) { d_det_pass<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
 // the same for replica blockIdx.y of a batch (parameter blocks PP[replica])
 template <int W, int SYS>
-__global__ void __launch_bounds__(kDetThreads, W == 8 ? 1 : 2) kb_det_pass(const Params* PP, const int* off, int R, int cur) {
+__global__ void __launch_bounds__(kDetThreads, W == 8 ? 2 : 4) kb_det_pass(const Params* PP, const int* off, int R, int cur) {
   __shared__ Params sP;
   __shared__ VGrid vg;
   if (!batch_block(PP, off, R, sP, vg)) return;
@@ -1378,7 +1383,7 @@ __device__ __forceinline__ void d_bucket(const Params& P, const VGrid vg) {
   if (st->error) return;
   const int64_t ns = st->nspawn < P.scap ? st->nspawn : P.scap, nb = st->nbuckets;
   // the det pass's look-back states, for the next iteration
-  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c < P.cap / kDetTile + 16; c += (int64_t)vg.n * blockDim.x)
+  for (int64_t c = (int64_t)vg.b * blockDim.x + threadIdx.x; c < P.cap / kDetTile + 33; c += (int64_t)vg.n * blockDim.x)
     P.det_state[c] = 0ull;
   for (int64_t s = (int64_t)vg.b * blockDim.x + threadIdx.x; s < ns; s += (int64_t)vg.n * blockDim.x) {
     const Key<W> k = load_key<W>(P.s_key, P.scap, s);

@@ -274,7 +274,7 @@ __device__ __forceinline__ void d_decide(const Params& P, int cur, const VGrid v
     }
     __syncthreads();
   }
-  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < nct + 16; i += (int64_t)vg.n * blockDim.x)
+  for (int64_t i = (int64_t)vg.b * blockDim.x + threadIdx.x; i < n / kDetTile + 33; i += (int64_t)vg.n * blockDim.x)
     P.det_state[i] = 0ull;   // look-back of the next det pass
   for (int64_t i = chunk_of(vg, wid, true) * 32 + lane; i < nu; i += (int64_t)vg.n * blockDim.x) {
     const int64_t s = P.u_spawn[i];
