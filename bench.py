@@ -127,46 +127,38 @@ def _peaks():
 def _phase_bytes(rec, W):
     """Algorithmic bytes per launch of the HBM-bound phases: K = 8W key bytes, a
     main-list entry is K + 17 bytes (key, int64 population, f64 diagonal, flag
-    byte), a bucketed spawn K + 9 (key, int64 amount, initiator byte), a staged
-    spawn K + 16 (key, amount, bucket/rank word)."""
+    byte), a staged spawn K + 16 (key, int64 amount, initiator/slot/position word)."""
     K = 8 * W
     ns, nd_pre, nd_post = float(rec["nspawn"]), float(rec["ndet_pre"]), float(rec["ndet"])
+    # staged spawns read once, main list read once, new list written once
+    merge = ns * (K + 16) + nd_pre * (K + 17) + nd_post * (K + 17)
     return {
-        # bucketed spawns read once, main list read once, new list written once
-        "merge": ns * (K + 9) + nd_pre * (K + 17) + nd_post * (K + 17),
-        # staged spawns read (key, amount, bucket/rank word), bucketed spawns written
-        "scatter": ns * (K + 16) + ns * (K + 9),
-        # main list read, populations/flags/attempt counts written
+        "merge": merge,
+        # main list read, populations/flags/attempt offsets written
         "det_pass": nd_pre * (K + 17) + nd_pre * (8 + 1 + 8),
-        # annihilation as a whole: spawns sorted (read + write) and merged (read),
-        # main list read, new list written
-        "annihilation": 3 * ns * (K + 9) + nd_pre * (K + 17) + nd_post * (K + 17),
+        "annihilation": merge,
         # whole iteration: the spawn and death phase (main list read, populations
         # and flags written, spawns written) plus the annihilation
-        "iteration": nd_pre * (K + 17) + nd_pre * 9 + ns * (K + 9)
-                     + 3 * ns * (K + 9) + nd_pre * (K + 17) + nd_post * (K + 17),
+        "iteration": nd_pre * (K + 17) + nd_pre * 9 + ns * (K + 16) + merge,
     }
 
 
 # Spawning kernel (k_attempt) issue-slot roofline.  Warp instructions issued
 # per spawn attempt and DRAM bytes per attempt, from one ncu capture of the
-# kernel on the profile case (profiles/kernels_molecule28_profile_case.md);
+# kernel on the profile case (profiles/kernels_molecule28_hash_path.md);
 # the peak is 4 warp instructions per cycle per SM (one per sub-partition) on
 # 152 SMs at the maximum SM clock.
-ATTEMPT_INST_PER_ATTEMPT = 235755617 / 7571203
-ATTEMPT_DRAM_BYTES_PER_ATTEMPT = (89.771008e6 + 7.630336e6) / 7571203
+ATTEMPT_INST_PER_ATTEMPT = 191147072 / 7571203
+ATTEMPT_DRAM_BYTES_PER_ATTEMPT = (90.750208e6 + 9.188352e6) / 7571203
 N_SM = 152
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of each phase's
 # kernels in the profile case's 4th iteration, and that iteration's counts
-# (profiles/traffic_molecule28_profile_case.md).  A phase's `traffic` in the
+# (profiles/kernels_molecule28_hash_path.md).  A phase's `traffic` in the
 # bench line is its ratio of these bytes to its algorithmic bytes times the
 # bench's own algorithmic bytes: both grow with the list and the spawns.
 PROFILE_CASE_REC = {"nspawn": 892485, "ndet_pre": 4040607, "ndet": 4031282}
-PROFILE_CASE_DRAM = {"det_pass": 101613056 + 22525952,
-                     "scatter": 23025408 + 1524736,
-                     "merge": (118296320 + 54569472) + (1056000 + 330240) + (109726464 + 49445888),
-                     "annihilation": 92928 + (23025408 + 1524736) + (118296320 + 54569472)
-                                     + (1056000 + 330240) + (109726464 + 49445888)}
+_MERGE_DRAM = ((77201920 + 2718720) + (76120832 + 4971264) + 15631872 + (106950144 + 56529152))   # match .. write
+PROFILE_CASE_DRAM = {"det_pass": 101775872 + 48205312, "merge": _MERGE_DRAM, "annihilation": _MERGE_DRAM}
 
 
 def _issue_peak():
@@ -242,7 +234,7 @@ def run_ours(args, rank, world):
     t_phase["annihilation"] = t_phase["bucket_scan"] + t_phase["scatter"] + t_phase["merge"]
     t_phase["iteration"] = t_max / args.steps
     byt_pc = _phase_bytes(PROFILE_CASE_REC, W)
-    for k in ("annihilation", "merge", "scatter", "det_pass", "iteration"):
+    for k in ("annihilation", "merge", "det_pass", "iteration"):
         t_s = t_phase[k] / 1e3
         ach = byt[k] / t_s / 1e9
         ratio = PROFILE_CASE_DRAM[k] / byt_pc[k] if k in PROFILE_CASE_DRAM else None
@@ -261,7 +253,7 @@ def run_ours(args, rank, world):
                     "ms_per_launch": round(ph["attempt"] / args.steps, 4),
                     "attempts_per_s": att_launch / t_att, "spawns_per_attempt": spawns_launch / att_launch,
                     "warp_instructions_per_spawn": ATTEMPT_INST_PER_ATTEMPT * att_launch / spawns_launch,
-                    "kernel": "k_attempt (spawning: Philox draw, excitation, spawn amount, bucket)",
+                    "kernel": "k_attempt (spawning: Philox draw, excitation, spawn amount)",
                     "per_unit": f"{ATTEMPT_INST_PER_ATTEMPT:.1f} warp instructions per attempt (ncu)",
                     "peak_source": f"4 warp instructions/cycle/SM x {N_SM} SMs x {imhz:.0f} MHz"}
 

@@ -199,7 +199,9 @@ hande_status hande_iterate(hande_ctx* ctx, int n);
  * (estimators, initiator flags, attempt counts, death), attempt-count scan,
  * bucket splitters, deterministic-space projection, spawning attempts,
  * bucket-count scan, bucket scatter, merge (annihilation), diagonal elements
- * of new determinants, shift/record. */
+ * of new determinants, shift/record.  The attempt-count scan is part of the
+ * determinant pass, and the default annihilation is all in `merge` (its new
+ * diagonals and the record included): those phases are then empty. */
 #define HANDE_NPHASES 10
 
 /* Advance n iterations like hande_iterate, but launched kernel by kernel

@@ -25,9 +25,12 @@
 //           entry's place follows from the keep bits and the survivors in front
 //           of it, a survivor's rank in its group from counting smaller keys.
 //           One thread closes the iteration meanwhile (shift, record).
-// What bounds them: match by L2 sectors and latency (one thread per spawn, all
-// resident), decide and write by HBM, the diagonal elements by the FP64 unit
-// (their sums are ordered), which runs beside the copy of the other blocks.
+// What bounds them: match by L1 passes (one 32-byte sector per lane and level) and
+// L2 latency, decide and write by HBM and latency, the diagonal elements by the
+// FP64 unit (their sums are ordered), which runs beside the copy of the other
+// blocks.  Measured in us, the bucket kernels they replace (scatter, warp and
+// block merges, scans, compaction, diagonals, record) -> these four: ueg 14e/38 at
+// 1e6 walkers 220 -> 72, molecule at 1e7 240 -> 142, hubbard 2d 18 at 2.2e6 310 -> 118.
 #pragma once
 
 namespace hande {
