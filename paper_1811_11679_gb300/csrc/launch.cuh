@@ -142,15 +142,19 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
   cudaStream_t aux = branch ? E.aux_stream : s;
   // captured iteration: the bucket split and the deterministic-space product
   // (they read only keys, the core populations and the CSR) run on a second
-  // branch beside the det pass.  The core update waits for the det pass, which
-  // reads the core populations, and runs beside the spawning, which does not
-  // read populations.  A failing record or wait invalidates the capture, which
+  // branch beside the det pass.  The spawning waits for the split, which clears
+  // the spawn counter.  The core update waits for the det pass, which reads the
+  // core populations, and runs beside the spawning, which does not read
+  // populations.  A failing record or wait invalidates the capture, which
   // ending the capture reports.
   if (branch) {
     (void)(cudaEventRecord(E.ev_fork, s));
     (void)(cudaStreamWaitEvent(aux, E.ev_fork, 0));
     if constexpr (kBuckets<W>)
-      if (!P.hash_merge) k_split<W><<<kScanBlocks, 256, 0, aux>>>(P, cur);
+      if (!P.hash_merge) {
+        k_split<W><<<kScanBlocks, 256, 0, aux>>>(P, cur);
+        (void)(cudaEventRecord(E.ev_join, aux));
+      }
     if (with_core) {
       k_core_locate<W><<<ncb, 256, 0, aux>>>(P, cur);
       k_core_spmv<<<spmv_blocks, 256, 0, aux>>>(P, cur);
@@ -160,6 +164,8 @@ void enqueue_iteration(Engine& E, int cur, bool core, cudaStream_t s, cudaEvent_
   k_det_pass<W, SYS><<<kScanBlocks, kDetThreads, 0, s>>>(P, cur);
   mark(1);
   mark(2);
+  // the spawning takes its staging slots from the counter that the split clears
+  if (branch && !P.hash_merge) (void)(cudaStreamWaitEvent(s, E.ev_join, 0));
   if (branch) {
     if (with_core) {
       (void)(cudaEventRecord(E.ev_fork, s));
@@ -263,13 +269,17 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
     (void)cudaEventRecord(fork, s);
     (void)cudaStreamWaitEvent(aux, fork, 0);
     if constexpr (kBuckets<W>)
-      if (!hash) kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
+      if (!hash) {
+        kb_split<W><<<blocks(0), 256, 0, aux>>>(PP, off(0), R, cur);
+        (void)cudaEventRecord(join, aux);
+      }
     if (G.max_ncore > 0) {
       kb_core_locate<W><<<dim3(ncb, R), 256, 0, aux>>>(PP, cur);
       kb_core_spmv<<<dim3((unsigned)(((int64_t)G.max_ncore * 32 + 255) / 256), R), 256, 0, aux>>>(PP, cur);
     }
   }
   kb_det_pass<W, SYS><<<blocks(0), kDetThreads, 0, s>>>(PP, off(0), R, cur);
+  if (branch && !hash) (void)cudaStreamWaitEvent(s, join, 0);   // the split clears the spawn counter
   if (branch) {
     if (G.max_ncore > 0) {
       (void)cudaEventRecord(fork, s);
