@@ -557,11 +557,14 @@ __device__ __forceinline__ void d_write(const Params& P, int cur, const VGrid vg
     }
   }
 }
+// Eight-word keys take more than 64 registers: held to two blocks per SM the
+// kernel spills 72 bytes (an iteration of ueg 14e/97 on 1.6e5 determinants 141
+// us, one block 136).
 template <int W, int SYS>
-__global__ void __launch_bounds__(kListThreads) k_write(Params P, int cur) { d_write<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
+__global__ void __launch_bounds__(kListThreads, W == 8 ? 1 : 2) k_write(Params P, int cur) { d_write<W, SYS>(P, cur, VGrid{(int)blockIdx.x, (int)gridDim.x}); }
 // the same for a replica of a batch (parameter blocks PP[replica])
 template <int W, int SYS>
-__global__ void __launch_bounds__(kListThreads) kb_write(const Params* PP, const int* off, int R, int cur) {
+__global__ void __launch_bounds__(kListThreads, W == 8 ? 1 : 2) kb_write(const Params* PP, const int* off, int R, int cur) {
   __shared__ Params sP;
   __shared__ VGrid vg;
   if (!batch_block(PP, off, R, sP, vg)) return;
