@@ -314,7 +314,9 @@ __device__ double h_double(const SysDev& s, const Key<W>& d, int i, int j, int a
   return ((n1 + n2) & 1) ? -v : v;
 }
 
-// <target|H|source> of two determinants that differ in two or four spin orbitals
+// <target|H|source> of two determinants that differ in two or four spin orbitals.
+// The number of differing orbitals decides, not of electrons moved: the estimator
+// of a caller's own list takes keys of any electron number.
 template <int W, int SYS>
 __device__ double h_connected(const SysDev& s, const Key<W>& src, const Key<W>& tgt) {
   Key<W> from, to;
@@ -324,10 +326,8 @@ __device__ double h_connected(const SysDev& s, const Key<W>& src, const Key<W>& 
     from.w[j] = x & src.w[j];
     to.w[j] = x & tgt.w[j];
   }
-  int nd = 0;
-#pragma unroll
-  for (int j = 0; j < W; ++j) nd += __popcll(from.w[j]);
-  if (nd == 1) return h_single<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(to, 0));
+  if (key_popc_xor<W>(src, tgt) == 2)
+    return h_single<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(to, 0));
   return h_double<W, SYS>(s, src, select_bit<W>(from, 0), select_bit<W>(from, 1), select_bit<W>(to, 0),
                           select_bit<W>(to, 1));
 }
