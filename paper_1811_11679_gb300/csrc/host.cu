@@ -1114,7 +1114,7 @@ hande_status hande_synchronize(hande_ctx* ctx) {
 }
 
 hande_status hande_estimators(hande_ctx* ctx, hande_estimate* out, int max, int* n_out) {
-  if (!ctx || (max > 0 && !out)) return HANDE_ERR_INVALID;
+  if (!ctx || max < 0 || (max > 0 && !out)) return HANDE_ERR_INVALID;
   Engine& E = ctx->E;
   if (n_out) *n_out = 0;
   if (E.failed) return HANDE_ERR_STATE;

@@ -1,5 +1,5 @@
-"""Order of an iteration's kernels, checked without a GPU: the library's object
-files linked against tests/_fakecuda.cpp, which records every launch with the
+"""Host code of the library without a GPU, above all the order of an iteration's
+kernels: its object files linked against tests/_fakecuda.cpp, which records every launch with the
 launches that streams and events put before it.  Kernels that share memory must
 be ordered on every annihilation path, for a single run and for a batch:
 
@@ -90,3 +90,15 @@ def test_batch(recorder, annihilation):
     b.iterate(2)
     _check_orders(recorder, BUCKETS if annihilation else HASH)
     b.close()
+
+
+def test_negative_record_count_is_refused(recorder):
+    """hande_estimators with max < 0 must not hand back records already fetched."""
+    g = hande.Hande(*_run(0), stream=1, torch_memory=False)
+    g.iterate(5)
+    n = C.c_int(7)
+    assert recorder.hande_estimators(g._h, None, -2, C.byref(n)) == -1
+    assert len(g.estimators()["iter"]) == 5
+    assert recorder.hande_estimators(g._h, None, -2, C.byref(n)) == -1
+    assert len(g.estimators()["iter"]) == 0
+    g.close()
