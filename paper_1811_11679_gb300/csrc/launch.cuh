@@ -212,7 +212,7 @@ void enqueue_buckets(Engine& E, int cur, cudaStream_t s, cudaEvent_t* ev) {
   auto mark = [&](int k) {
     if (ev) cudaEventRecord(ev[k], s);
   };
-  k_bucket<W><<<E.attempt_grid * 4, 256, 0, s>>>(P);
+  k_bucket<W><<<E.attempt_grid * 4, 256, 0, s>>>(P, cur);
   int64_t* nbk = st_field_i64(st, offsetof(DevState, nbuckets));
   k_scan_one<uint32_t, uint32_t><<<1, 1024, 0, s>>>(P.bcount, P.boff, nbk,
                                                     st_field_i64(st, offsetof(DevState, scan_total)), -1, st);
@@ -298,7 +298,7 @@ void enqueue_iteration_batch(BatchGroup& G, int cur, cudaStream_t s, cudaStream_
     return;
   }
   if constexpr (kBuckets<W>) {
-  kb_bucket<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
+  kb_bucket<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R, cur);
   kb_scan_buckets<<<dim3(1, R), 1024, 0, s>>>(PP);
   kb_scatter<W><<<blocks(2), 256, 0, s>>>(PP, off(2), R);
   if (E0.merge_warp) {
