@@ -20,6 +20,7 @@ import subprocess
 import pytest
 
 from paper_1811_11679_gb300 import build, hande, inputs
+from test_gpu_tc_gemm_paths import SHAPES
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 BUCKETS = [("det_pass", "attempt"), ("split", "attempt"), ("split", "bucket"), ("attempt", "bucket"),
@@ -102,3 +103,12 @@ def test_negative_record_count_is_refused(recorder):
     assert recorder.hande_estimators(g._h, None, -2, C.byref(n)) == -1
     assert len(g.estimators()["iter"]) == 0
     g.close()
+
+
+@pytest.mark.parametrize("width,m,n,k,ldd,shift", SHAPES)
+def test_gemm_tile_width(recorder, width, m, n, k, ldd, shift):
+    recorder.fake_reset()
+    pad = (k + 7) // 8 * 8
+    assert recorder.hande_gemm_bf16(4096, pad, 8192, pad, 4 * shift + 16384, ldd, m, n, k, 512, 1) == 0
+    name = recorder.fake_name(recorder.fake_count() - 1).decode()
+    assert f"k_gemm_bf16_tn_pILi{width}ELi0E" in name
