@@ -231,6 +231,8 @@ def run_ours(args, rank, world):
     byt = _phase_bytes(per, W)
     roof = {}
     t_phase = {k: ph[k] / args.steps for k in ph}
+    # the default annihilation is all in `merge`: the two differ by the empty phases'
+    # events only, and their bytes are the same
     t_phase["annihilation"] = t_phase["bucket_scan"] + t_phase["scatter"] + t_phase["merge"]
     t_phase["iteration"] = t_max / args.steps
     byt_pc = _phase_bytes(PROFILE_CASE_REC, W)

@@ -183,10 +183,11 @@ typedef struct hande_ctx hande_ctx;
 hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, const hande_allocator* allocator,
                                void* cuda_stream, hande_ctx** out);
 
-/* Advance n >= 0 iterations (asynchronous; one CUDA-graph launch per iteration).
- * Errors of an iteration surface at the next synchronising call.  With
- * annihilation 1 or 2 the annihilation
- * buckets are sized from the previous iteration's spawn and new-key counts; a
+/* Advance n >= 0 iterations (asynchronous; one CUDA-graph launch for four
+ * iterations while nothing on the host is due between them -- online training,
+ * a running time-step search, the choice of the deterministic space -- else one
+ * per iteration).  Errors of an iteration surface at the next synchronising
+ * call.  With annihilation 1 or 2 the annihilation buckets are sized from the previous iteration's spawn and new-key counts; a
  * bucket that still receives more spawns than one warp takes is split into at
  * most 256 key sub-ranges of about a quarter tile each (splitters sampled from
  * its spawns), so one list entry whose spawns in a single iteration exceed
@@ -213,7 +214,7 @@ hande_status hande_iterate_timed(hande_ctx* ctx, int n, float* phase_ms, int nph
 /* Wait for the stream and report latched device errors. */
 hande_status hande_synchronize(hande_ctx* ctx);
 
-/* Copy the records not yet fetched (oldest first, at most `max`) to `out`;
+/* Copy the records not yet fetched (oldest first, at most `max` >= 0) to `out`;
  * *n_out = records written.  Synchronises.  HANDE_ERR_CAPACITY if records
  * were overwritten before being fetched (record_capacity too small). */
 hande_status hande_estimators(hande_ctx* ctx, hande_estimate* out, int max, int* n_out);

@@ -124,7 +124,7 @@ bool same_group(const Engine& a, const Engine& c) {
 // Block budgets of each group's phases: `scale` times the single run's grid
 // for that phase (the planner divides them among the replicas by their work);
 // a replica never gets more than 4 single-run grids, nor more list-pass blocks
-// than its scan partials hold.
+// than a single run's det pass (four per SM).
 void set_grids(hande_batch* b) {
   const double f = b->scale > 0.0 ? b->scale : 2.0;
   for (auto& G : b->groups) {

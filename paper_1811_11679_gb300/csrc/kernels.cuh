@@ -3,8 +3,8 @@
 // sort the spawned array and merge it into the sorted main list).
 //
 //   det_pass      per determinant: projected-energy terms (App. A.1), initiator
-//                 flag (Sec. 2.1), spawning-attempt count, death/cloning
-//   scan          exclusive scan of attempt counts (attempt space)
+//                 flag (Sec. 2.1), spawning-attempt counts and their scan (attempt
+//                 space), death/cloning
 //   core_*        semi-stochastic exact projection inside the deterministic space
 //   attempt       per attempt: Philox draw, excitation, H_ij, spawn amount
 //   match, decide, place, write   the default annihilation (merge_hash.cuh)
@@ -422,9 +422,9 @@ __device__ __forceinline__ unsigned long long lookback_warp(DevState* st, unsign
 // matrix elements evaluated by full warps while warp 0 looks back.
 // Bound: Philox issue and the FP64 unit (death: five operations per entry) at half
 // occupancy.  Four blocks of 256 threads per SM instead of two of 512, so that
-// others run while one waits at its look-back: one pass of ueg 14e/38 3293 ->
-// 3231 us, proposal table 1821 -> 1783, hubbard 2d 18 4984 -> 4902, molecule 1e7
-// 14184 -> 14053.
+// others run while one waits at its look-back.  In us per report block (20 whole
+// iterations, the records and the list): ueg 14e/38 3293 -> 3231, proposal table
+// 1821 -> 1783, hubbard 2d 18 4984 -> 4902, molecule 1e7 14184 -> 14053.
 constexpr int kDetThreads = 256;
 constexpr int kDetItems = 2;
 constexpr int kDetTile = kDetThreads * kDetItems;   // 512
@@ -981,7 +981,6 @@ static __global__ void kb_core_apply(const Params* PP, int cur) {
   d_core_apply(sP, cur);
 }
 
-// ------------------------------------------------------------------ attempts
 // ------------------------------------------------------------------ attempts
 // Attempts are processed 32 per warp.  Most draws come to nothing (target
 // orbitals occupied or outside the basis), so the rest of an attempt goes through

@@ -1,7 +1,7 @@
 // launch.cuh -- per-(key width, system) launchers: the iteration sequence, the
 // deterministic-space selection ("high" space, HANDE-QMC paper App. A.2) and
 // the CSR build of the deterministic-space Hamiltonian.  Included once per key
-// width by inst_w{1,2,8}.cu so the three widths compile in parallel.
+// width by inst_w{1,2,3,8}.cu so the four widths compile in parallel.
 #pragma once
 #include <cstddef>
 

@@ -252,8 +252,11 @@ __device__ __forceinline__ void epi_store(const Epilogue& ep, const uint32_t (&r
 constexpr int kPThreads = 192;
 // FP32 output staged per epilogue warp: two buffers of 32 x 32 values, stored by
 // TMA (128-byte swizzle).  Lanes hold rows of the accumulator, so direct stores
-// put the 32 lanes of an instruction into 32 rows, 16 bytes each; the layer of
-// the 246-orbital table refresh (121088 x 256 x 512) went from 61 to 47 us.
+// put the 32 lanes of an instruction into 32 rows, 16 bytes each; a product of
+// 121088 x 256 x 512 went from 61 to 47 us.  Of the learned proposal's own
+// products the two hidden gradients take it; its hidden layers leave through the
+// BF16 epilogue, its weight gradients in parts, and its logits have rows that do
+// not end on 16 bytes (38 or 246 columns): those are stored directly.
 constexpr uint32_t kOutBytes = 32 * 32 * 4;
 constexpr uint32_t kOutWarpBytes = 2 * kOutBytes;
 // tensor-memory columns (two FP32 accumulators of BN columns: 512 at BN = 256)
