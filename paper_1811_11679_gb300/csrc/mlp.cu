@@ -78,14 +78,14 @@ int sm_count(int dev) {
 
 // persistent launch: one CTA per SM (at most one per output tile)
 template <int BN, int EPI>
-bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md, int tma_out, const Epilogue& ep,
-                  int M, int N, int K, unsigned* err, cudaStream_t s, int dev, int nsm, const char** why) {
+bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md, const Epilogue& ep, int M,
+                  int N, int K, unsigned* err, cudaStream_t s, int dev, int nsm, const char** why) {
   static bool attr_set[256] = {};
   {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!attr_set[dev]) {
       if (cudaFuncSetAttribute(k_gemm_bf16_tn_p<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)PTile<BN>::kSmemBytes) != cudaSuccess) {
+                               (int)PTile<BN, EPI>::kSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         *why = "cannot reserve the GEMM's shared memory";
         return false;
@@ -95,7 +95,7 @@ bool launch_shape(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMa
   }
   const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + kBM - 1) / kBM) * (ep.parts > 1 ? ep.parts : 1);
   const unsigned grid = (unsigned)(tiles < nsm ? tiles : nsm);
-  k_gemm_bf16_tn_p<BN, EPI><<<grid, kPThreads, PTile<BN>::kSmemBytes, s>>>(ma, mb, md, tma_out, ep, M, N, K, err);
+  k_gemm_bf16_tn_p<BN, EPI><<<grid, kPThreads, PTile<BN, EPI>::kSmemBytes, s>>>(ma, mb, md, ep, M, N, K, err);
   if (cudaGetLastError() != cudaSuccess) {
     *why = "GEMM launch failed";
     return false;
@@ -134,18 +134,20 @@ bool launch_gemm_ep(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t l
   while (bn > 64 && tm * ((N + bn - 1) / bn) * (ep.parts > 1 ? ep.parts : 1) < nsm) bn >>= 1;
   CUtensorMap ma, mb, md{};
   // (a TMA store clips a row in 16-byte steps, so N is a multiple of 4 too)
-  const int tma_out = epi == EPI_F32 && ep.parts <= 1 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) && !(N & 3) ? 1 : 0;
+  const bool tma_out = epi == EPI_F32 && ep.parts <= 1 && !((uintptr_t)ep.D & 15) && !(ep.ldd & 3) && !(N & 3);
   if (!make_map(&ma, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, kBM) ||
       !make_map(&mb, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, (uint32_t)bn) ||
       (tma_out && !make_out_map(&md, ep.D, (uint64_t)N, (uint64_t)M, (uint64_t)ep.ldd))) {
     *why = "cuTensorMapEncodeTiled failed";
     return false;
   }
-  auto go = [&](auto launch) { return launch(ma, mb, md, tma_out, ep, M, N, K, err, s, dev, nsm, why); };
-  if (epi == EPI_F32)
-    return go(bn == 256 ? &launch_shape<256, EPI_F32> : (bn == 128 ? &launch_shape<128, EPI_F32> : &launch_shape<64, EPI_F32>));
-  return go(bn == 256 ? &launch_shape<256, EPI_BF16_BIAS>
-                      : (bn == 128 ? &launch_shape<128, EPI_BF16_BIAS> : &launch_shape<64, EPI_BF16_BIAS>));
+  auto go = [&](auto l256, auto l128, auto l64) {
+    return (bn == 256 ? l256 : (bn == 128 ? l128 : l64))(ma, mb, md, ep, M, N, K, err, s, dev, nsm, why);
+  };
+  if (tma_out)
+    return go(&launch_shape<256, EPI_F32_TMA>, &launch_shape<128, EPI_F32_TMA>, &launch_shape<64, EPI_F32_TMA>);
+  if (epi == EPI_F32) return go(&launch_shape<256, EPI_F32>, &launch_shape<128, EPI_F32>, &launch_shape<64, EPI_F32>);
+  return go(&launch_shape<256, EPI_BF16_BIAS>, &launch_shape<128, EPI_BF16_BIAS>, &launch_shape<64, EPI_BF16_BIAS>);
 }
 
 bool launch_gemm(const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb, float* D, int64_t ldd, int M,

@@ -46,7 +46,8 @@ struct Tile {
 };
 // epilogues: FP32 D, or BF16 act(D + bias) (ReLU or none) with an optional
 // transposed BF16 copy
-enum { EPI_F32 = 0, EPI_BF16_BIAS = 1 };
+// (EPI_F32_TMA: EPI_F32 stored by TMA, chosen by launch_gemm_ep)
+enum { EPI_F32 = 0, EPI_BF16_BIAS = 1, EPI_F32_TMA = 2 };
 struct Epilogue {
   float* D;                 // EPI_F32: D[row * ldd + col]
   int64_t ldd;
@@ -261,27 +262,33 @@ constexpr uint32_t kOutBytes = 32 * 32 * 4;
 constexpr uint32_t kOutWarpBytes = 2 * kOutBytes;
 // tensor-memory columns (two FP32 accumulators of BN columns: 512 at BN = 256)
 // and dynamic shared memory (1024-byte aligned stages + barriers)
-template <int BN>
+// (only the kernel that stores through it has the staging buffer and its code: in
+// every kernel they took the table refresh of 246 orbitals, whose logits are
+// stored directly, from 316 to 323 us; 313 without)
+template <int BN, int EPI>
 struct PTile {
   static constexpr uint32_t kTmemCols = 2 * BN;
   static constexpr size_t kStageBytes = (size_t)kStages * (kTileABytes + Tile<BN>::kTileBBytes);
-  static constexpr size_t kSmemBytes = 1024 + kStageBytes + 4 * kOutWarpBytes + 256;
+  // (at 64 columns always, which also keeps to one CTA per SM: with two sizes of
+  // shared memory among its products the learner's gradients took 183 us instead
+  // of 180, the kernels' own times unchanged)
+  static constexpr size_t kOutTotal = EPI == EPI_F32_TMA || BN == 64 ? 4 * (size_t)kOutWarpBytes : 0;
+  static constexpr size_t kSmemBytes = 1024 + kStageBytes + kOutTotal + 256;
 };
 
 template <int BN, int EPI>
 __global__ void __launch_bounds__(kPThreads, 1)
     k_gemm_bf16_tn_p(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                     const __grid_constant__ CUtensorMap tmD, int tma_out, const Epilogue ep, int M, int N, int K,
-                     unsigned* err) {
+                     const __grid_constant__ CUtensorMap tmD, const Epilogue ep, int M, int N, int K, unsigned* err) {
   constexpr uint32_t kTileBBytes = Tile<BN>::kTileBBytes;
-  constexpr uint32_t kTmemCols = PTile<BN>::kTmemCols;
+  constexpr uint32_t kTmemCols = PTile<BN, EPI>::kTmemCols;
   extern __shared__ __align__(16) unsigned char tcp_smem_raw[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tcp_smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = base;
   unsigned char* sB = base + (size_t)kStages * kTileABytes;
-  unsigned char* sOut = base + PTile<BN>::kStageBytes;   // 1024-byte aligned
-  uint64_t* full = reinterpret_cast<uint64_t*>(sOut + 4 * kOutWarpBytes);
+  unsigned char* sOut = base + PTile<BN, EPI>::kStageBytes;   // 1024-byte aligned
+  uint64_t* full = reinterpret_cast<uint64_t*>(sOut + PTile<BN, EPI>::kOutTotal);
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;      // [2]
   uint64_t* acc_empty = acc_full + 2;        // [2]
@@ -294,6 +301,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const int tn_count = (N + BN - 1) / BN, tm_count = (M + kBM - 1) / kBM;
   const int parts = ep.parts > 1 ? ep.parts : 1, per = parts > 1 ? ep.part_chunks : nk;
   const int nout = tn_count * tm_count, ntiles = nout * parts;   // work items: part-major
+  // (no division where K is not divided: it stands before a tile's first load and
+  // before its stores, 0.7 of 17.8 us at 20000 x 130 x 64)
+  auto part_of = [&](int t) { return parts > 1 ? t / nout : 0; };
 
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -324,8 +334,8 @@ __global__ void __launch_bounds__(kPThreads, 1)
       int64_t fill = 0;   // chunk loads issued over all tiles
       int64_t landed = 0;
       for (int t = (int)blockIdx.x; t < ntiles && !s_fail; t += (int)gridDim.x) {
-        const int o = t % nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
-        const int k0 = t / nout * per, k1 = k0 + per < nk ? k0 + per : nk;
+        const int p = part_of(t), o = t - p * nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
+        const int k0 = p * per, k1 = k0 + per < nk ? k0 + per : nk;
         for (int kc = k0; kc < k1 && !s_fail; ++kc, ++fill) {
           const int st = (int)(fill % kStages);
           const uint32_t ph = (uint32_t)((fill / kStages) & 1);
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         }
         tc_fence_after();
         const uint32_t dcol = tmem + (uint32_t)(a * BN);
-        const int k0 = t / nout * per, k1 = k0 + per < nk ? k0 + per : nk;
+        const int k0 = part_of(t) * per, k1 = k0 + per < nk ? k0 + per : nk;
         for (int kc = k0; kc < k1; ++kc, ++use) {
           const int st = (int)(use % kStages);
           if (!mbar_wait(&full[st], (uint32_t)((use / kStages) & 1))) {
@@ -384,9 +394,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
     uint32_t stores = 0;
     int i = 0;
     for (int t = (int)blockIdx.x; t < ntiles && !s_fail; t += (int)gridDim.x, ++i) {
-      const int o = t % nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
+      const int p = part_of(t), o = t - p * nout, m0 = (o / tn_count) * kBM, n0 = (o % tn_count) * BN;
       Epilogue pe = ep;
-      pe.D += (int64_t)(t / nout) * ep.part_stride;
+      if (EPI == EPI_F32) pe.D += p * ep.part_stride;
       const int a = i & 1;
       const bool ok = mbar_wait(&acc_full[a], (uint32_t)((i >> 1) & 1));
       if (!__all_sync(0xffffffffu, ok)) {   // warp-uniform (the accumulator reads are warp-collective)
@@ -399,7 +409,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if (n0 + c0 >= N) break;
         uint32_t r[32];
         tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * BN + c0), r);
-        if (EPI == EPI_F32 && tma_out) {
+        if (EPI == EPI_F32_TMA) {
           if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // this buffer was read
           __syncwarp();
           unsigned char* b = out + (stores++ & 1) * kOutBytes + lane * 128;
@@ -421,7 +431,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[a]);
     }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (EPI == EPI_F32_TMA && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();

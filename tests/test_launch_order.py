@@ -106,9 +106,10 @@ def test_negative_record_count_is_refused(recorder):
 
 
 @pytest.mark.parametrize("width,m,n,k,ldd,shift", SHAPES)
-def test_gemm_tile_width(recorder, width, m, n, k, ldd, shift):
+def test_gemm_tile_width_and_store_path(recorder, width, m, n, k, ldd, shift):
     recorder.fake_reset()
     pad = (k + 7) // 8 * 8
     assert recorder.hande_gemm_bf16(4096, pad, 8192, pad, 4 * shift + 16384, ldd, m, n, k, 512, 1) == 0
     name = recorder.fake_name(recorder.fake_count() - 1).decode()
-    assert f"k_gemm_bf16_tn_pILi{width}ELi0E" in name
+    tma = shift % 4 == 0 and ldd % 4 == 0 and n % 4 == 0   # the kernel with the staged TMA store (2), or without (0)
+    assert f"k_gemm_bf16_tn_pILi{width}ELi{2 if tma else 0}E" in name
