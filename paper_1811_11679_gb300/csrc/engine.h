@@ -68,13 +68,39 @@ struct Ops {
 // kernels were measured beside it and left out: they gained nothing on top and
 // cost the long iterations 3%.
 constexpr int kGraphIters = 4;
-constexpr int kPinRecords = 64;   // records read back through the page-locked block
+constexpr int kPinRecords = 64;   // records read back through the host block
 constexpr int kPhases = 10;   // timed phases of one iteration
 
 Ops ops_w1(int kind);
 Ops ops_w2(int kind);
 Ops ops_w3(int kind);
 Ops ops_w8(int kind);
+
+// Host memory of small transfers.  Page-locked memory makes them direct (a report's
+// records and state 10 us sooner) but takes 100 us to get and 160 to give back,
+// three times the rest of creating and destroying a small context, so a block
+// becomes page-locked after kPinAfter uses; an object of few calls never pays.
+constexpr int kPinAfter = 16;
+struct HostBlock {
+  std::vector<char> page;
+  void* pin = nullptr;
+  int uses = 0;
+  // the block (every call with the same size); earlier addresses stay valid
+  char* get(size_t bytes) {
+    if (!pin && uses++ == kPinAfter && cudaHostAlloc(&pin, bytes, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();   // ordinary memory serves as well
+      pin = nullptr;
+    }
+    if (pin) return static_cast<char*>(pin);
+    if (uses > kPinAfter) uses = kPinAfter + 1;
+    if (page.empty()) page.resize(bytes);
+    return page.data();
+  }
+  void release() {   // no copy may be in flight
+    if (pin) cudaFreeHost(pin);
+    pin = nullptr;
+  }
+};
 
 struct Engine {
   Params P{};            // device pointers and run constants (kernel argument)
@@ -114,7 +140,7 @@ struct Engine {
   unsigned* check_word = nullptr;   // result word of the walker-list checks
   int64_t core_table_cap = 0;
   double e_ref = 0.0;
-  void* pin = nullptr;              // page-locked host block: DevState, then kPinRecords records
+  HostBlock host;                   // DevState, then kPinRecords records
   // UEG proposal table (excit_gen = 1): cumulative weights on the device and
   // the drawable mask (host and device); the learned proposal, if attached
   uint32_t* ptab = nullptr;

@@ -45,8 +45,7 @@ void release_all(Engine& E) {
     cudaStreamDestroy(E.aux_stream);
     E.aux_stream = nullptr;
   }
-  if (E.pin) cudaFreeHost(E.pin);
-  E.pin = nullptr;
+  E.host.release();
   if (E.ev_fork) cudaEventDestroy(E.ev_fork);
   if (E.ev_join) cudaEventDestroy(E.ev_join);
   E.ev_fork = E.ev_join = nullptr;
@@ -426,18 +425,18 @@ void set_tau(Engine& E, double tau, bool to_device) {
                        cudaMemcpyHostToDevice, E.stream));
 }
 
-// The device state in the page-locked block, after the stream's work (and after
-// any copies the caller enqueued before this): one synchronisation.  Reading
-// its words one by one into pageable memory cost a synchronisation each, about
-// 10 us of the host's time.
+// The device state in the host block, after the stream's work (and after any
+// copies the caller enqueued before this): one synchronisation.  Reading its
+// words one by one cost a synchronisation each, about 10 us of the host's time.
+constexpr size_t kHostState = (sizeof(DevState) + 63) & ~size_t(63);
+char* host_block(Engine& E) { return E.host.get(kHostState + kPinRecords * sizeof(Record)); }
 const DevState& read_state(Engine& E) {
-  CK(cudaMemcpyAsync(E.pin, E.P.st, sizeof(DevState), cudaMemcpyDeviceToHost, E.stream));
+  char* b = host_block(E);
+  CK(cudaMemcpyAsync(b, E.P.st, sizeof(DevState), cudaMemcpyDeviceToHost, E.stream));
   CK(cudaStreamSynchronize(E.stream));
-  return *static_cast<const DevState*>(E.pin);
+  return *reinterpret_cast<const DevState*>(b);
 }
-Record* pin_records(Engine& E) {
-  return reinterpret_cast<Record*>(static_cast<char*>(E.pin) + ((sizeof(DevState) + 63) & ~size_t(63)));
-}
+Record* pin_records(Engine& E) { return reinterpret_cast<Record*>(host_block(E) + kHostState); }
 
 unsigned read_error(Engine& E) { return read_state(E).error; }
 
@@ -914,8 +913,6 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
     sd.ptab_cum = nullptr;
     if (q.excit_gen == 1) proposal_init(E, T.kvec.data(), T.klookup.data(), sd.nmax, sd.side);
 
-    CK(cudaHostAlloc(&E.pin, ((sizeof(DevState) + 63) & ~size_t(63)) + kPinRecords * sizeof(Record), cudaHostAllocDefault));
-
     // ---- device buffers
     const int64_t cap = P.cap, scap = P.scap;
     for (int b = 0; b < 2; ++b) {
@@ -941,7 +938,6 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       P.hash_size = 1024;
       while (P.hash_size < 2 * (uint64_t)scap && P.hash_size < (1ull << 31)) P.hash_size <<= 1;
       P.hash_tab = dalloc<uint32_t>(E, P.hash_size);
-      CK(cudaMemsetAsync(P.hash_tab, 0, P.hash_size * sizeof(uint32_t), E.stream));
       P.u_spawn = dalloc<uint32_t>(E, scap);
       P.u_rank = dalloc<uint32_t>(E, scap);
       P.n_pos = dalloc<uint32_t>(E, scap);
@@ -953,8 +949,16 @@ hande_status hande_init_system(const hande_system* sys, const hande_qmc* qmc, co
       P.t_base = dalloc<unsigned long long>(E, tiles);
       P.occ_draw = dalloc<uint32_t>(E, cap);
       P.core_move = dalloc<uint32_t>(E, cap);
-      for (int l = 1; l < kEndLevels && (cap >> (2 * l)) > 0; ++l)
-        P.s_end[l] = dalloc<uint64_t>(E, (size_t)end_stride(cap, l) * E.W);
+      // (one allocation for the levels: twelve took 25 us of the 180 that creating and
+      // destroying a small context takes)
+      size_t ends = 0;
+      for (int l = 1; l < kEndLevels && (cap >> (2 * l)) > 0; ++l) ends += (size_t)end_stride(cap, l) * E.W;
+      uint64_t* end = dalloc<uint64_t>(E, ends);
+      for (int l = 1; l < kEndLevels && (cap >> (2 * l)) > 0; ++l) {
+        P.s_end[l] = end;
+        end += (size_t)end_stride(cap, l) * E.W;
+      }
+      CK(cudaMemsetAsync(P.hash_tab, 0, P.hash_size * sizeof(uint32_t), E.stream));
     } else {
       P.b_flag = dalloc<uint8_t>(E, scap);
       P.bcount = dalloc<uint32_t>(E, cap);

@@ -63,7 +63,7 @@ struct Learner {
   int32_t *in_rows = nullptr, *in_tgt = nullptr;
   float* in_w = nullptr;
   float* probs = nullptr;
-  char* pin = nullptr;   // page-locked: a batch's rows, targets and weights, then the loss and the error word
+  HostBlock host;        // a batch's rows, targets and weights, then the loss and the error word
   cudaGraphExec_t graph = nullptr;
 };
 
@@ -607,7 +607,6 @@ void learner_attach(Engine& E, const hande_learning& in) {
   L.in_rows = dalloc<int32_t>(E, 3 * (size_t)L.S);   // one upload for the three
   L.in_tgt = L.in_rows + L.S;
   L.in_w = reinterpret_cast<float*>(L.in_tgt + L.S);
-  CK(cudaHostAlloc((void**)&L.pin, 12 * (size_t)L.S + 16, cudaHostAllocDefault));
   L.probs = dalloc<float>(E, (size_t)L.S * M);
   // sample buffers of the spawning kernel
   E.P.smp_row = dalloc<int32_t>(E, L.S);
@@ -646,9 +645,9 @@ void learner_attach(Engine& E, const hande_learning& in) {
 void learner_release(Engine& E) {
   if (!E.learn) return;
   if (E.learn->graph) cudaGraphExecDestroy(E.learn->graph);
-  if (E.learn->pin) {
+  if (E.learn->host.pin) {
     cudaStreamSynchronize(E.stream);
-    cudaFreeHost(E.learn->pin);
+    E.learn->host.release();
   }
   delete E.learn;
   E.learn = nullptr;
@@ -670,12 +669,15 @@ void learner_params(Engine& E, float* get, const float* set) {
   CK(cudaStreamSynchronize(E.stream));
 }
 
+static char* host_block(Learner& L) { return L.host.get(12 * (size_t)L.S + 16); }
+
 // upload a batch of n <= S samples (rows, targets, weights; the rest weight 0)
-// through the page-locked block, one copy (the calls that use it synchronise
-// before they return, so the block is free again)
+// through the host block, one copy (the calls that use it synchronise before they
+// return, so the block is free again; one that fails leaves the context unusable)
 static void upload_batch(Engine& E, Learner& L, const int32_t* rows, const int32_t* tgt, const float* w, int n) {
   const int R = L.R, M = L.M;
-  int32_t* r = reinterpret_cast<int32_t*>(L.pin);
+  char* block = host_block(L);
+  int32_t* r = reinterpret_cast<int32_t*>(block);
   int32_t* t = r + L.S;
   float* ww = reinterpret_cast<float*>(t + L.S);
   for (int i = 0; i < n; ++i) {
@@ -690,11 +692,11 @@ static void upload_batch(Engine& E, Learner& L, const int32_t* rows, const int32
   std::memset(r + n, 0, sizeof(int32_t) * (size_t)(L.S - n));
   std::memset(t + n, 0, sizeof(int32_t) * (size_t)(L.S - n));
   std::memset(ww + n, 0, sizeof(float) * (size_t)(L.S - n));
-  CK(cudaMemcpyAsync(L.in_rows, L.pin, 12 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
+  CK(cudaMemcpyAsync(L.in_rows, block, 12 * (size_t)L.S, cudaMemcpyHostToDevice, E.stream));
 }
 // the loss and the error word of the stream's work (synchronises)
 static double read_loss(Engine& E, Learner& L) {
-  char* p = L.pin + 12 * (size_t)L.S;
+  char* p = host_block(L) + 12 * (size_t)L.S;
   CK(cudaMemcpyAsync(p, L.loss, 16, cudaMemcpyDeviceToHost, E.stream));
   CK(cudaStreamSynchronize(E.stream));
   unsigned e;

@@ -30,6 +30,7 @@ struct Config {
   cudaStream_t stream;
 } config;
 uintptr_t next_handle = 16;
+int host_allocs = 0, device_allocs = 0;   // page-locked blocks held, device allocations since the reset
 template <class T>
 cudaError_t make(T* h) {
   *h = reinterpret_cast<T>(next_handle += 16);
@@ -49,7 +50,9 @@ CUresult encode_tiled(CUtensorMap* m, ...) {
 
 extern "C" {
 // ---- what a test asks
-void fake_reset() { launches.clear(), done.clear(); }
+void fake_reset() { launches.clear(), done.clear(), device_allocs = 0; }
+int fake_host_allocs() { return host_allocs; }
+int fake_device_allocs() { return device_allocs; }
 int fake_count() { return (int)launches.size(); }
 const char* fake_name(int i) { return launches[i].name.c_str(); }
 int fake_before(int a, int b) { return (int)launches[b].before.count(a); }
@@ -92,10 +95,10 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
 }
 
 // ---- the rest succeeds
-cudaError_t cudaMalloc(void** p, size_t n) { return alloc(p, n); }
-cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return alloc(p, n); }
+cudaError_t cudaMalloc(void** p, size_t n) { return ++device_allocs, alloc(p, n); }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return ++host_allocs, alloc(p, n); }
 cudaError_t cudaFree(void* p) { return free(p), cudaSuccess; }
-cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) { return --host_allocs, free(p), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
   return std::memcpy(d, s, n), cudaSuccess;
 }

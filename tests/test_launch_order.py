@@ -113,3 +113,17 @@ def test_gemm_tile_width_and_store_path(recorder, width, m, n, k, ldd, shift):
     name = recorder.fake_name(recorder.fake_count() - 1).decode()
     tma = shift % 4 == 0 and ldd % 4 == 0 and n % 4 == 0   # the kernel with the staged TMA store (2), or without (0)
     assert f"k_gemm_bf16_tn_pILi{width}ELi{2 if tma else 0}E" in name
+
+
+def test_creating_a_context_page_locks_nothing(recorder):
+    """The host block of the read-backs becomes page-locked with use, once."""
+    recorder.fake_reset()
+    g = hande.Hande(*_run(0), stream=1, torch_memory=False)
+    assert recorder.fake_host_allocs() == 0
+    assert recorder.fake_device_allocs() < 60
+    for _ in range(40):
+        g.iterate(1)
+        assert len(g.estimators()["iter"]) == 1
+    assert recorder.fake_host_allocs() == 1
+    g.close()
+    assert recorder.fake_host_allocs() == 0
