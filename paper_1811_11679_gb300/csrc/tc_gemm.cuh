@@ -419,10 +419,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0 && m0 + warp * 32 < M) {   // rows and columns beyond D are clipped
-            tma_store_2d(&tmD, b, n0 + c0, m0 + warp * 32);
+          if (lane == 0) {   // rows and columns beyond D are clipped
+            if (m0 + warp * 32 < M) tma_store_2d(&tmD, b, n0 + c0, m0 + warp * 32);
+            // a group for every chunk, empty past the last row too: the wait above
+            // counts groups, and without it the second chunk of such a tile was
+            // written over the buffer that the tile before still stored from
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
           }
+          __syncwarp();
         } else {
           epi_store<EPI>(pe, r, m0 + lrow, n0, c0, M, N);
         }

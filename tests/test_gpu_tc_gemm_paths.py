@@ -47,3 +47,26 @@ def test_width_and_store_path(width, m, n, k, ldd, shift):
     assert torch.all((d.double() - exact).abs() <= bound)
     d.fill_(7.0)
     assert torch.all(flat == 7.0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m,n,k", [(128 * 38 + 8, 2048, 64), (128 * 152 + 96, 252, 64), (128 * 304 + 1, 252, 72)])
+def test_last_tile_past_the_rows_leaves_the_tile_before_alone(m, n, k):
+    """CTAs that walk a whole tile and then one with warps wholly past M, which
+    store nothing, many times over (the error bound as above)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g = torch.Generator(device="cuda").manual_seed(m)
+    a = torch.randn((m, k), generator=g, device="cuda").to(torch.bfloat16)
+    b = torch.randn((n, k), generator=g, device="cuda").to(torch.bfloat16)
+    exact = a.double() @ b.double().T
+    bound = 4.0 * k * 2.0 ** -24 * (a.double().abs() @ b.double().abs().T) + 1e-30
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(200):
+        d = hande.gemm_bf16(a, b, status=status)
+        bad += ((d.double() - exact).abs() > bound).sum()
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    assert bad.item() == 0
