@@ -15,56 +15,83 @@ namespace hande {
 // zero adds nothing to the exact product).  Hubbard and UEG elements are mostly
 // zero at that distance (no bond, momentum not conserved), so only nonzero ones
 // are kept: on the 18-site cluster the product went from 65 to 11 us.
-template <int W, int SYS>
-__device__ __forceinline__ double core_elem(const Params& P, int r, int c, const Key<W>& kr, const Key<W>& kc) {
-  if (r == c) return __dsub_rn(h_diag<W, SYS>(P.sys, kr), P.st->e_ref);
-  return h_elem<W, SYS>(P.sys, kc, kr);
-}
-template <int W, int SYS>
-__device__ __forceinline__ bool core_stored(const Params& P, int r, int c, const Key<W>& kr, const Key<W>& kc) {
-  const int nd = key_popc_xor<W>(kr, kc);
-  if (SYS == SYS_MOLECULE || nd == 0) return nd <= 4;
-  if (SYS == SYS_HUBBARD ? nd != 2 : nd != 4) return false;
-  return nonzero(h_connected<W, SYS>(P.sys, kc, kr));
-}
-template <int W, int SYS>
-__global__ void k_csr_count(Params P, int32_t* rowcnt) {
-  int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (r >= P.ncore) return;
-  Key<W> kr = load_key<W>(P.core_key, P.ncore, r);
-  int cnt = 0;
+// One warp per row.  Columns that differ in the right number of orbitals (a few
+// percent) are queued and their elements evaluated 32 at a time by full warps, in
+// ascending order: evaluated where they were found, nearly every step of 32
+// columns waited for one element.  Choosing the space, in ms: ueg 14e/38 of 2e4
+// determinants 2.57 -> 2.12, ueg 14e/66 of 3e3 1.05 -> 0.77, molecule of 3e4 5.1 ->
+// 2.9 (1.83, 1.00 and 5.2 while zero elements were kept).
+constexpr int kCsrThreads = 256;
+constexpr int kCsrQueue = 64;   // holds 31 + 32 columns
+// (DIAG: the diagonal element is wanted, not only its place)
+template <int W, int SYS, bool DIAG, class Emit>
+__device__ __forceinline__ void csr_row(const Params& P, int r, const Key<W>& kr, int* queue, Emit emit) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;
+  auto flush = [&](int take) {   // the first `take` queued columns
+    bool keep = false;
+    int c = 0;
+    double h = 0.0;
+    if (lane < take) {
+      c = queue[lane];
+      if (c != r) h = h_connected<W, SYS>(P.sys, load_key<W>(P.core_key, P.ncore, c), kr);
+      else if (DIAG) h = __dsub_rn(h_diag<W, SYS>(P.sys, kr), P.st->e_ref);
+      keep = SYS == SYS_MOLECULE || c == r || nonzero(h);
+    }
+    emit(__ballot_sync(0xffffffffu, keep), keep, c, h);
+    n -= take;
+    __syncwarp();
+    if (lane < n) queue[lane] = queue[take + lane];   // only after a full step: n < 32
+    __syncwarp();
+  };
   for (int c0 = 0; c0 < P.ncore; c0 += 32) {
-    int c = c0 + lane;
-    bool nz = false;
-    if (c < P.ncore) nz = core_stored<W, SYS>(P, r, c, kr, load_key<W>(P.core_key, P.ncore, c));
-    cnt += __popc(__ballot_sync(0xffffffffu, nz));
+    const int c = c0 + lane;
+    bool near = false;
+    if (c < P.ncore) {
+      const int nd = key_popc_xor<W>(kr, load_key<W>(P.core_key, P.ncore, c));
+      near = nd == 0 || (SYS == SYS_MOLECULE ? nd <= 4 : nd == (SYS == SYS_HUBBARD ? 2 : 4));
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, near);
+    if (near) queue[n + __popc(m & ((1u << lane) - 1u))] = c;
+    n += __popc(m);
+    __syncwarp();
+    if (n >= 32) flush(32);
+  }
+  if (n > 0) flush(n);
+}
+template <int W, int SYS>
+__global__ void __launch_bounds__(kCsrThreads) k_csr_count(Params P, int32_t* rowcnt) {
+  __shared__ int queue[kCsrThreads / 32][kCsrQueue];
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (r >= P.ncore) return;
+  const Key<W> kr = load_key<W>(P.core_key, P.ncore, r);
+  int cnt = 0;
+  if (SYS == SYS_MOLECULE) {   // every near pair is kept
+    for (int c0 = 0; c0 < P.ncore; c0 += 32) {
+      const int c = c0 + lane;
+      const bool near = c < P.ncore && key_popc_xor<W>(kr, load_key<W>(P.core_key, P.ncore, c)) <= 4;
+      cnt += __popc(__ballot_sync(0xffffffffu, near));
+    }
+  } else {
+    csr_row<W, SYS, false>(P, r, kr, queue[threadIdx.x >> 5], [&](unsigned m, bool, int, double) { cnt += __popc(m); });
   }
   if (lane == 0) rowcnt[r] = cnt;
 }
 template <int W, int SYS>
-__global__ void k_csr_fill(Params P, int64_t* rowptr, int32_t* col, double* val) {
-  int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kCsrThreads) k_csr_fill(Params P, int64_t* rowptr, int32_t* col, double* val) {
+  __shared__ int queue[kCsrThreads / 32][kCsrQueue];
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (r >= P.ncore) return;
-  Key<W> kr = load_key<W>(P.core_key, P.ncore, r);
+  const Key<W> kr = load_key<W>(P.core_key, P.ncore, r);
   int64_t o = rowptr[r];
-  for (int c0 = 0; c0 < P.ncore; c0 += 32) {
-    int c = c0 + lane;
-    bool conn = false;
-    Key<W> kc;
-    if (c < P.ncore) {
-      kc = load_key<W>(P.core_key, P.ncore, c);
-      conn = core_stored<W, SYS>(P, r, c, kr, kc);
-    }
-    unsigned m = __ballot_sync(0xffffffffu, conn);
-    if (conn) {
-      int64_t e = o + __popc(m & ((1u << lane) - 1u));
+  csr_row<W, SYS, true>(P, r, kr, queue[threadIdx.x >> 5], [&](unsigned m, bool keep, int c, double h) {
+    if (keep) {
+      const int64_t e = o + __popc(m & ((1u << lane) - 1u));
       col[e] = c;
-      val[e] = core_elem<W, SYS>(P, r, c, kr, kc);
+      val[e] = h;
     }
     o += __popc(m);
-  }
+  });
 }
 // ------------------------------------------------------------------ selection of the core
 template <int W>
